@@ -50,7 +50,8 @@ __global__ void __launch_bounds__(256, 3) sweep_batch_kernel(const BatchArgs p) 
       ctr3 = (PURPOSE_MOVE << 24) | (S.g.replica & 0xFFFFFFu);
       TN = S.G * S.g.N;
     }
-    auto lane_ok = [&](uint32_t t) { return t < S.full_tiles || L.li0 < S.last_rows; };
+    auto lane_ok = [&](uint32_t t) { return L.in_tile(t < S.full_tiles, S.last_rows); };
+    const uint32_t dense_tiles = TN == 64u ? S.full_tiles : 0u;   // no masks needed
     const uint32_t t0 = it.t0 + warp;
     float2 px = make_float2(0.f, 0.f), py = px, pz = px;
     if (t0 < it.t1 && lane_ok(t0)) {
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(256, 3) sweep_batch_kernel(const BatchArgs p) 
         py = __ldcs(reinterpret_cast<const float2*>(S.y + bn));
         pz = __ldcs(reinterpret_cast<const float2*>(S.z + bn));
       }
-      if (tile < S.full_tiles)
+      if (tile < dense_tiles)
         my_acc += pair_tile<WT, uint32_t, false, false>(S.g, p.keys, L, S.x, S.y, S.z, nacc, base, base,
                                                  true, sweep, ctr3, S.set_order_random, S.a, S.K_b, x0,
                                                  x1, y0, y1, z0, z1);

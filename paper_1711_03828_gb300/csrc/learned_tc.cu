@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(128) sweep_learned_tc_kernel(const SweepArgs p
   const uint32_t TN = p.G * p.g.N;
   unsigned my_acc = 0;
   for (uint32_t tile = t_begin + wib; tile < t_end; tile += 4) {
-    const bool valid = tile < (uint32_t)p.full_tiles || L.li0 < p.last_rows;
+    const bool valid = L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
     my_acc += learned_pair_tile<WT, WarpNet>(p, L, net, nacc, tile * TN + L.li0, valid, sweep, A0, A1);
   }
 #pragma unroll
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(128) sweep_learned_umma_kernel(const SweepArgs
   unsigned my_acc = 0;
   for (uint32_t r = 0; r < rounds; ++r) {
     const uint32_t tile = t_begin + 4 * r + (uint32_t)wib;
-    const bool valid = tile < t_end && (tile < (uint32_t)p.full_tiles || L.li0 < p.last_rows);
+    const bool valid = tile < t_end && L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
     const uint32_t base = (tile < t_end ? tile : t_begin) * TN + L.li0;
     my_acc += learned_pair_tile<WT, UmmaNet>(p, L, net, nacc, base, valid && net.ok, sweep, A0, A1);
   }

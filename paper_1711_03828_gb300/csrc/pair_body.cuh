@@ -31,6 +31,8 @@ struct PairLane {
   const WT* w1;
   uint32_t v0, v1;
   uint32_t li0;
+  uint32_t tile_rows;   // particles of a full tile, N * floor(64/N): 64 when N divides 64, else
+                        // fewer, and the last lanes hold no pair of this tile
   uint32_t ci0;         // chain position of slot 0
   uint32_t lane_chain;  // chain of this lane within the tile
 
@@ -38,6 +40,7 @@ struct PairLane {
                                        const void* wB) {
     lane = lane_;
     li0 = 2u * (uint32_t)lane;
+    tile_rows = (64u / N) * N;
     ci0 = li0 % N;                                // chain position of slot 0 (even)
     lane_chain = li0 / N;
     first_lane = (int)((li0 - ci0) >> 1);         // lane holding the chain's particle 0
@@ -48,6 +51,11 @@ struct PairLane {
     src_prev = (lane - 1) & 31;
     src_next = (lane + 1) & 31;
     set_types(ci0 >= N_A, ci0 + 1u >= N_A, wA, wB);
+  }
+
+  // Whether this lane's pair belongs to a full tile, or to the last one of last_rows particles.
+  __device__ __forceinline__ bool in_tile(bool full, uint32_t last_rows) const {
+    return li0 < (full ? tile_rows : last_rows);
   }
 
   // Types of the two slots (true: B): field planes and count increments.

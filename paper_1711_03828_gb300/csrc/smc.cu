@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
   // positions of the warp's next tile, loaded while the current one is moved
   float2 nx = make_float2(0.f, 0.f), ny = nx, nz = nx;
   auto load_pos = [&](uint32_t t) {
-    if (t < t_end && (t < (uint32_t)p.full_tiles || L.li0 < p.last_rows)) {
+    if (t < t_end && L.in_tile(t < (uint32_t)p.full_tiles, p.last_rows)) {
       const uint32_t b = t * TN + L.li0;
       nx = __ldcs(reinterpret_cast<const float2*>(p.x + b));
       ny = __ldcs(reinterpret_cast<const float2*>(p.y + b));
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
   uint32_t tile = claim();
   load_pos(tile);
   while (tile < t_end) {
-    const bool valid = tile < (uint32_t)p.full_tiles || L.li0 < p.last_rows;
+    const bool valid = L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
     const uint32_t base = tile * TN + L.li0;
     float2 px = make_float2(0.f, 0.f), py = px, pz = px;
     if (valid) {

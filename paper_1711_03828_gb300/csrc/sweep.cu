@@ -246,7 +246,9 @@ __global__ void __launch_bounds__(768, 1) sweep_pair_kernel(const SweepArgs p) {
   L.init(lane, p.g.N, p.g.N_A, p.wA, p.wB);
   const uint32_t TN = p.G * p.g.N;
   const uint32_t full_tiles = (uint32_t)p.full_tiles;
-  auto lane_ok = [&](uint32_t t) { return t < full_tiles || L.li0 < p.last_rows; };
+  auto lane_ok = [&](uint32_t t) { return L.in_tile(t < full_tiles, p.last_rows); };
+  // tiles that fill all 64 slots need no masks
+  const uint32_t dense_tiles = TN == 64u ? full_tiles : 0u;
   const bool wide = p.g.nx > 1 && p.g.ny > 1 && p.g.nz > 1;
 
   float2 px = make_float2(0.f, 0.f), py = px, pz = px;
@@ -274,11 +276,11 @@ __global__ void __launch_bounds__(768, 1) sweep_pair_kernel(const SweepArgs p) {
       Lt.set_types((seq >> L.ci0) & 1ull, (seq >> (L.ci0 + 1u)) & 1ull, p.wA, p.wB);
     }
     const IDX cbase = base + (IDX)p.g.id_base;
-    if (tile < full_tiles && wide)
+    if (tile < dense_tiles && wide)
       my_acc += pair_tile<WT, IDX, false, true>(p.g, p.g, Lt, p.x, p.y, p.z, nacc, base, cbase, true,
                                                 sweep, ctr3, p.set_order_random, p.a, p.K_b, x0, x1,
                                                 y0, y1, z0, z1);
-    else if (tile < full_tiles)
+    else if (tile < dense_tiles)
       my_acc += pair_tile<WT, IDX, false, false>(p.g, p.g, Lt, p.x, p.y, p.z, nacc, base, cbase, true,
                                                  sweep, ctr3, p.set_order_random, p.a, p.K_b, x0,
                                                  x1, y0, y1, z0, z1);
