@@ -598,7 +598,7 @@ soma_status soma_batch_get_timing(soma_batch_t* b, soma_timing* out);
  * out:      host array of k doubles; returns after the results are there.
  * stream:   cudaStream_t to run on (NULL: legacy default stream).
  *
- * Scratch (twiddle tables and block partial sums, about 768 KB) lives in one
+ * Scratch (twiddle tables and block partial sums, about 272 KB) lives in one
  * file-scope device array of libsoma.  The first call on each device sets it
  * up: it looks up the array's device address, and with CUDA's lazy module
  * loading (the default) that lookup is what loads this part of the library

@@ -69,6 +69,7 @@ constexpr uint32_t GRAPH_CHUNK = 16;
 constexpr uint64_t MAX_M = 1ull << 40;
 // Supported position range |x|, |y|, |z| < 2^18 dL (exact cell fold).
 constexpr uint64_t POS_LIMIT = 1ull << 18;
+constexpr size_t SQ_CALL_MAX = 4096;   // wave vectors of one structure factor call
 
 }  // namespace
 
@@ -119,8 +120,7 @@ struct soma_t {
   int topo_grid = 1;
   double* d_out = nullptr;
   size_t scratch_doubles = 0;
-  double* d_tw = nullptr;
-  size_t tw_doubles = 0;
+  double* d_tw = nullptr;                    // S(q): twiddles of the axes, results (lazy)
   SweepShape shape;
   uint64_t host_sweep = 0;
   uint64_t launches = 0;
@@ -1242,7 +1242,7 @@ soma_status structure_factor_of(soma_t* h, const uint32_t* nn, const int32_t* m,
 soma_status soma_structure_factor(soma_t* h, const int32_t* m, size_t k, double* out) {
   if (!h || !m || !out) return fail(SOMA_EINVAL, "NULL argument");
   if (h->n_types) return fail(SOMA_EINVAL, "n_t types: use soma_structure_factor_types");
-  if (k > 4096) return fail(SOMA_EINVAL, "k=%zu > 4096", k);
+  if (k > SQ_CALL_MAX) return fail(SOMA_EINVAL, "k=%zu > %zu", k, SQ_CALL_MAX);
   if (k == 0) return SOMA_OK;
   return structure_factor_of(h, h->n[h->host_sweep & 1], m, k, out);
 }
@@ -1253,7 +1253,7 @@ soma_status soma_structure_factor_types(soma_t* h, uint32_t ti, uint32_t tj, con
   const uint32_t T = h->n_types ? h->n_types : 2u;
   if (ti >= T || tj >= T || ti == tj)
     return fail(SOMA_EINVAL, "types %u, %u: need two different types below %u", ti, tj, T);
-  if (k > 4096) return fail(SOMA_EINVAL, "k=%zu > 4096", k);
+  if (k > SQ_CALL_MAX) return fail(SOMA_EINVAL, "k=%zu > %zu", k, SQ_CALL_MAX);
   if (k == 0) return SOMA_OK;
   // two types: the packed A | B grid (S of B - A equals S of A - B)
   if (!h->n_types) return structure_factor_of(h, h->n[h->host_sweep & 1], m, k, out);
@@ -1274,43 +1274,38 @@ soma_status soma_structure_factor_types(soma_t* h, uint32_t ti, uint32_t tj, con
 namespace {
 soma_status structure_factor_of(soma_t* h, const uint32_t* nn, const int32_t* m, size_t k,
                                 double* out) {
-  const int nx = h->g.nx, ny = h->g.ny, nz = h->g.nz;
-  const size_t T = (size_t)nx + ny + nz;
-  const size_t need = (size_t)SQ_MAX * T * 2;
-  if (h->tw_doubles < need) {
-    cudaFree(h->d_tw);
-    h->d_tw = nullptr;
-    SOMA_CUDA(cudaMalloc((void**)&h->d_tw, sizeof(double) * need));
-    h->tw_doubles = need;
+  const int n3[3] = {h->g.nx, h->g.ny, h->g.nz};
+  const size_t T = (size_t)n3[0] + n3[1] + n3[2];
+  if (!h->d_tw) {   // the axes' twiddles and room for the results, once per handle
+    double* d = nullptr;
+    SOMA_CUDA(cudaMalloc((void**)&d, sizeof(double) * (2 * T + SQ_CALL_MAX)));
+    std::vector<double> tw(2 * T);
+    const double two_pi = 6.283185307179586;
+    size_t off = 0;
+    for (int a = 0; a < 3; ++a)
+      for (int r = 0; r < n3[a]; ++r) {
+        const double ph = two_pi * (double)r / (double)n3[a];
+        tw[off++] = std::cos(ph);
+        tw[off++] = -std::sin(ph);
+      }
+    cudaError_t e = cudaMemcpyAsync(d, tw.data(), sizeof(double) * 2 * T, cudaMemcpyHostToDevice,
+                                    h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);   // tw leaves scope
+    if (e != cudaSuccess) {
+      cudaFree(d);
+      return cuda_fail(e, "S(q) twiddles");
+    }
+    h->d_tw = d;
   }
-  std::vector<double> tw(need);
-  const double two_pi = 6.283185307179586;
+  double* res = h->d_tw + 2 * T;
   for (size_t q0 = 0; q0 < k; q0 += SQ_MAX) {
     const int kk = (int)((k - q0) < (size_t)SQ_MAX ? (k - q0) : (size_t)SQ_MAX);
-    for (int q = 0; q < kk; ++q) {
-      const int n3[3] = {nx, ny, nz};
-      size_t off = (size_t)q * T * 2;
-      for (int d = 0; d < 3; ++d) {
-        const long long md = m[3 * (q0 + q) + d];
-        for (int c = 0; c < n3[d]; ++c) {
-          long long r = (md * c) % n3[d];
-          if (r < 0) r += n3[d];
-          const double ph = two_pi * (double)r / (double)n3[d];
-          tw[off++] = std::cos(ph);
-          tw[off++] = -std::sin(ph);
-        }
-      }
-    }
-    SOMA_CUDA(cudaMemcpyAsync(h->d_tw, tw.data(), sizeof(double) * kk * T * 2,
-                              cudaMemcpyHostToDevice, h->stream));
-    SOMA_CUDA(launch_structure_factor(h->g, nn, h->d_tw, kk, h->d_scratch, h->d_out, h->stream));
+    SOMA_CUDA(launch_structure_factor(h->g, nn, h->d_tw, m + 3 * q0, kk, h->d_scratch, res + q0,
+                                      h->stream));
     h->launches += 2;
-    SOMA_CUDA(cudaMemcpyAsync(out + q0, h->d_out, sizeof(double) * kk, cudaMemcpyDeviceToHost,
-                              h->stream));
-    soma_status st = sync(h);
-    if (st != SOMA_OK) return st;
   }
-  return SOMA_OK;
+  SOMA_CUDA(cudaMemcpyAsync(out, res, sizeof(double) * k, cudaMemcpyDeviceToHost, h->stream));
+  return sync(h);
 }
 }  // namespace
 

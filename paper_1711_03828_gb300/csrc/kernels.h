@@ -65,12 +65,14 @@ cudaError_t launch_observables(const Geom& g, const float* x, const float* y, co
                                int hamiltonian, const float* ext, double* part, double* out,
                                cudaStream_t st);
 
-// S(q) for k <= SQ_MAX wave vectors; tw holds per q the FP64 twiddles
-// (cos, sin) of the three axes, laid out [q][nx + ny + nz][2].
+// S(q) for k <= SQ_MAX wave vectors m (host, k x 3); tw (device) holds the FP64
+// twiddles e^{-2 pi i r/n} (cos, -sin), r < n, of the three axes in turn
+// (nx + ny + nz pairs); part: SQ_BLOCKS * 2 * SQ_MAX doubles of scratch.
 constexpr int SQ_MAX = 32;
 constexpr int SQ_BLOCKS = 512;
-cudaError_t launch_structure_factor(const Geom& g, const uint32_t* n, const double* tw, int k,
-                                    double* part, double* out, cudaStream_t st);
+cudaError_t launch_structure_factor(const Geom& g, const uint32_t* n, const double* tw,
+                                    const int32_t* m, int k, double* part, double* out,
+                                    cudaStream_t st);
 
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, size_t n,
                           cudaStream_t st);

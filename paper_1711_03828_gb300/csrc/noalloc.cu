@@ -20,37 +20,26 @@ namespace {
 
 constexpr int NOALLOC_MAX_K = SOMA_SQ_NOALLOC_MAX_K;         // wave vectors per call
 constexpr int NOALLOC_MAX_AXES = SOMA_SQ_NOALLOC_MAX_AXES;   // grid_x + grid_y + grid_z
-constexpr size_t TW_DOUBLES = (size_t)NOALLOC_MAX_K * NOALLOC_MAX_AXES * 2;
+constexpr size_t TW_DOUBLES = (size_t)NOALLOC_MAX_AXES * 2;
 constexpr size_t PART_DOUBLES = (size_t)SQ_BLOCKS * 2 * SQ_MAX;
 constexpr size_t OUT_DOUBLES = SQ_MAX;
 static_assert(NOALLOC_MAX_K <= SQ_MAX, "one reduction launch per call");
 
-// twiddles | block partial sums | results  (about 768 KB)
+// twiddles | block partial sums | results  (about 272 KB)
 static __device__ __align__(256) double g_sq_scratch[TW_DOUBLES + PART_DOUBLES + OUT_DOUBLES];
 
-struct WaveVectors {
-  int32_t m[3 * NOALLOC_MAX_K];
-};
-
-// e^{-2 pi i m c / n} per axis, in FP64, with the argument reduced exactly
-// (m c mod n in integers) before sincospi.
-__global__ void twiddle_kernel(const WaveVectors wv, int k, int nx, int ny, int nz,
-                               double* __restrict__ tw) {
+// The axes' twiddles e^{-2 pi i r/n}, r < n, in FP64.
+__global__ void twiddle_kernel(int nx, int ny, int nz, double* __restrict__ tw) {
   const int T = nx + ny + nz;
-  const int total = k * T;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += gridDim.x * blockDim.x) {
-    const int q = idx / T, t = idx - q * T;
-    int d, c, n;
-    if (t < nx) { d = 0; c = t; n = nx; }
-    else if (t < nx + ny) { d = 1; c = t - nx; n = ny; }
-    else { d = 2; c = t - nx - ny; n = nz; }
-    long long r = ((long long)wv.m[3 * q + d] * c) % n;
-    if (r < 0) r += n;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < T; idx += gridDim.x * blockDim.x) {
+    int r, n;
+    if (idx < nx) { r = idx; n = nx; }
+    else if (idx < nx + ny) { r = idx - nx; n = ny; }
+    else { r = idx - nx - ny; n = nz; }
     double sn, cs;
     sincospi(2.0 * (double)r / (double)n, &sn, &cs);
-    tw[2 * (size_t)idx] = cs;
-    tw[2 * (size_t)idx + 1] = -sn;
+    tw[2 * idx] = cs;
+    tw[2 * idx + 1] = -sn;
   }
 }
 
@@ -102,13 +91,10 @@ extern "C" soma_status soma_structure_factor_noalloc(const soma_system_desc* des
   double* tw = base;
   double* part = base + TW_DOUBLES;
   double* res = part + PART_DOUBLES;
-  WaveVectors wv;
-  for (size_t i = 0; i < 3 * k; ++i) wv.m[i] = m[i];
   const cudaStream_t s = (cudaStream_t)stream;
-  const int total = (int)k * (g.nx + g.ny + g.nz);
-  twiddle_kernel<<<(total + 255) / 256, 256, 0, s>>>(wv, (int)k, g.nx, g.ny, g.nz, tw);
+  twiddle_kernel<<<(g.nx + g.ny + g.nz + 127) / 128, 128, 0, s>>>(g.nx, g.ny, g.nz, tw);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_structure_factor(g, density, tw, (int)k, part, res, s);
+  if (e == cudaSuccess) e = launch_structure_factor(g, density, tw, m, (int)k, part, res, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double) * k, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return report_cuda(e, "soma_structure_factor_noalloc");
