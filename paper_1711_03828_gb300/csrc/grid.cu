@@ -6,6 +6,7 @@
 //   - energies: Eq. (h-bond), (V-harmonic), (discrete-ham); S(q): Sec. 5.6.
 #include "kernels.h"
 #include "draws.cuh"
+#include "square_sum.cuh"
 
 namespace soma {
 
@@ -276,26 +277,14 @@ cudaError_t launch_sort_chains(const Geom& g, const float* src, uint64_t src_pla
 }
 
 // ---------------------------------------------------------------------------
-// FP64 block reduction in a fixed order (deterministic for a fixed launch).
-template <int K>
-__device__ __forceinline__ void block_sum(double (&v)[K], double* sh /* K*32 */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
-  if (lane == 0)
-    for (int k = 0; k < K; ++k) sh[k * 32 + wid] = v[k];
-  __syncthreads();
-  if (wid == 0) {
-    const int nw = blockDim.x >> 5;
-    for (int k = 0; k < K; ++k) {
-      double t = lane < nw ? sh[k * 32 + lane] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-      v[k] = t;
-    }
-  }
-}
-
+// Sums over bonds |b|^2 and over chains |R_e|^2 (square_sum.cuh).
+//
+// One thread per particle; the positions are read once from memory (a bond's
+// upper particle hits the line of the next lane).  With the squares in FP64 the
+// kernel was bound by that pipe (two lanes per SM and cycle, 87 % busy, and the
+// one chain end in a warp cost it a whole warp's operations): 748 us for 16.8M
+// particles.  With the kernels below the analysis of that melt (64 wave
+// vectors) went from 1.48 to 0.57 ms.
 __global__ void __launch_bounds__(256) chain_obs_kernel(const Geom g, const float* __restrict__ x,
                                                         const float* __restrict__ y,
                                                         const float* __restrict__ z,
@@ -303,21 +292,21 @@ __global__ void __launch_bounds__(256) chain_obs_kernel(const Geom g, const floa
   __shared__ double sh[2 * 32];
   const uint64_t M = g.n_chains * g.N;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  double v[2] = {0.0, 0.0};
-  for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < M; m += stride) {
-    const uint32_t i = (uint32_t)(m % g.N);
-    const double x0 = x[m], y0 = y[m], z0 = z[m];
-    if (i + 1 < g.N) {
-      const double dx = (double)x[m + 1] - x0, dy = (double)y[m + 1] - y0,
-                   dz = (double)z[m + 1] - z0;
-      v[0] += dx * dx + dy * dy + dz * dz;
+  const uint32_t N = g.N, step = (uint32_t)(stride % N);
+  uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t i = (uint32_t)(m % N);
+  SquareSum bonds, ends;
+  for (; m < M; m += stride) {
+    const float x0 = x[m], y0 = y[m], z0 = z[m];
+    if (i + 1u < N) bonds.add(x[m + 1], y[m + 1], z[m + 1], x0, y0, z0);
+    if (i == 0u) {
+      const uint64_t e = m + N - 1u;
+      ends.add(x[e], y[e], z[e], x0, y0, z0);
     }
-    if (i == 0) {
-      const uint64_t e = m + g.N - 1;
-      const double dx = (double)x[e] - x0, dy = (double)y[e] - y0, dz = (double)z[e] - z0;
-      v[1] += dx * dx + dy * dy + dz * dz;
-    }
+    i += step;
+    if (i >= N) i -= N;
   }
+  double v[2] = {bonds.value(), ends.value()};
   block_sum<2>(v, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x * 2 + 0] = v[0];
@@ -325,57 +314,101 @@ __global__ void __launch_bounds__(256) chain_obs_kernel(const Geom g, const floa
   }
 }
 
+// Energy of the occupation numbers.  With rho = rho_0 dL^3, r = round(rho) and
+// the integers d = n_A + n_B - r and f = n_A - n_B, a cell's energy is
+//   kappaN/2 (d + r - rho)^2/rho^2 - chiN/4 f^2/rho^2     (K^0; K^1: + chiN n_A n_B/rho^2),
+// so the sums of d, d^2 and f^2 (or n_A n_B) over a block's cells are taken as
+// exact integers and combined in FP64 once per block: no FP64 operation per
+// cell (39 us before at 96^3 cells), and the squares of the deviations are
+// summed without cancellation.  The external energy, if any, is summed in FP64.
 __global__ void __launch_bounds__(256) grid_obs_kernel(const Geom g, const uint32_t* __restrict__ n,
                                                        double inv_rho, double kappaN, double chiN,
                                                        int hamiltonian, const float* __restrict__ ext,
                                                        double* __restrict__ part) {
-  __shared__ double sh[2 * 32];
-  double v[2] = {0.0, 0.0}, e_ext = 0.0;
+  __shared__ double sh[32];
+  __shared__ long long si[3][8];
+  __shared__ uint32_t sm[2][8];
+  const double rho = 1.0 / inv_rho;
+  const long long r = llrint(rho < 131072.0 ? rho : 131072.0);   // counts stay below 2^17
+  long long s1 = 0, s2 = 0, s3 = 0;
+  uint32_t mx = 0u, cnt = 0u;
+  double e_ext[1] = {0.0};
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < g.cells; c += stride) {
     const uint32_t w = n[c];
-    const double a = (double)(w & 0xFFFFu), b = (double)(w >> 16);
-    const double phiA = a * inv_rho, phiB = b * inv_rho;
-    const double fl = phiA + phiB - 1.0, df = phiA - phiB;
-    v[0] += hamiltonian ? 0.5 * kappaN * fl * fl + chiN * phiA * phiB
-                        : 0.5 * kappaN * fl * fl - 0.25 * chiN * df * df;
-    if (ext) e_ext += a * (double)ext[c] + b * (double)ext[g.cells + c];
-    v[1] = fmax(v[1], a + b);
+    const uint32_t a = w & 0xFFFFu, b = w >> 16;
+    const int d = (int)(a + b) - (int)r, f = (int)a - (int)b;
+    s1 += d;
+    s2 += (long long)d * d;
+    s3 += hamiltonian ? (long long)a * b : (long long)f * f;
+    mx = max(mx, a + b);
+    ++cnt;
+    if (ext) e_ext[0] += (double)a * (double)ext[c] + (double)b * (double)ext[g.cells + c];
   }
-  // the max is folded by a second pass over the per-warp maxima
-  double mx = v[1];
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, o));
-  __shared__ double shm[32];
-  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = mx;
-  double s1[2] = {v[0], e_ext};
-  block_sum<2>(s1, sh);
+  for (int o = 16; o > 0; o >>= 1) {
+    s1 += __shfl_xor_sync(FULL, s1, o);
+    s2 += __shfl_xor_sync(FULL, s2, o);
+    s3 += __shfl_xor_sync(FULL, s3, o);
+    mx = max(mx, __shfl_xor_sync(FULL, mx, o));
+    cnt += __shfl_xor_sync(FULL, cnt, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    const int k = threadIdx.x >> 5;
+    si[0][k] = s1;
+    si[1][k] = s2;
+    si[2][k] = s3;
+    sm[0][k] = mx;
+    sm[1][k] = cnt;
+  }
+  if (ext) block_sum<1>(e_ext, sh);   // uniform: ext is a kernel argument
+  __syncthreads();
   if (threadIdx.x == 0) {
-    double m2 = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m2 = fmax(m2, shm[k]);
-    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 0] = s1[0];
-    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 1] = m2;
-    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 2] = s1[1];
+    s1 = s2 = s3 = 0;
+    mx = cnt = 0u;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
+      s1 += si[0][k];
+      s2 += si[1][k];
+      s3 += si[2][k];
+      mx = max(mx, sm[0][k]);
+      cnt += sm[1][k];
+    }
+    const double off = (double)r - rho;
+    const double fl = (double)s2 + off * (2.0 * (double)s1 + off * (double)cnt);
+    const double K = inv_rho * inv_rho *
+                     (0.5 * kappaN * fl + (hamiltonian ? chiN : -0.25 * chiN) * (double)s3);
+    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 0] = K;
+    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 1] = (double)mx;
+    part[2 * OBS_BLOCKS + blockIdx.x * 3 + 2] = e_ext[0];
   }
 }
 
-__global__ void obs_final_kernel(const double* __restrict__ part, int nb_chain, int nb_grid,
-                                 double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double b2 = 0.0, re2 = 0.0, k = 0.0, mx = 0.0, ee = 0.0;
-  for (int i = 0; i < nb_chain; ++i) {
-    b2 += part[2 * i];
-    re2 += part[2 * i + 1];
+// Folds the blocks' sums in a fixed order, one block of threads instead of one
+// thread (306 us before with 1024 blocks each, the FP64 additions and their
+// loads one after another).
+__global__ void __launch_bounds__(256) obs_final_kernel(const double* __restrict__ part, int nb_chain,
+                                                        int nb_grid, double* __restrict__ out) {
+  __shared__ double sh[4 * 32];
+  __shared__ double shm[8];
+  double v[4] = {0.0, 0.0, 0.0, 0.0}, mx = 0.0;
+  for (int i = threadIdx.x; i < nb_chain; i += 256) {
+    v[0] += part[2 * i];
+    v[1] += part[2 * i + 1];
   }
-  for (int i = 0; i < nb_grid; ++i) {
-    k += part[2 * OBS_BLOCKS + 3 * i];
+  for (int i = threadIdx.x; i < nb_grid; i += 256) {
+    v[2] += part[2 * OBS_BLOCKS + 3 * i];
     mx = fmax(mx, part[2 * OBS_BLOCKS + 3 * i + 1]);
-    ee += part[2 * OBS_BLOCKS + 3 * i + 2];
+    v[3] += part[2 * OBS_BLOCKS + 3 * i + 2];
   }
-  out[0] = b2;
-  out[1] = re2;
-  out[2] = k;
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, o));
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = mx;
+  block_sum<4>(v, sh);
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) mx = fmax(mx, shm[k]);
+  out[0] = v[0];
+  out[1] = v[1];
+  out[2] = v[2];
   out[3] = mx;
-  out[4] = ee;
+  out[4] = v[3];
 }
 
 cudaError_t launch_observables(const Geom& g, const float* x, const float* y, const float* z,
@@ -390,7 +423,7 @@ cudaError_t launch_observables(const Geom& g, const float* x, const float* y, co
   chain_obs_kernel<<<(unsigned)nb1, 256, 0, st>>>(g, x, y, z, part);
   grid_obs_kernel<<<(unsigned)nb2, 256, 0, st>>>(g, n, inv_rho, kappaN, chiN, hamiltonian, ext,
                                                  part);
-  obs_final_kernel<<<1, 32, 0, st>>>(part, (int)nb1, (int)nb2, out);
+  obs_final_kernel<<<1, 256, 0, st>>>(part, (int)nb1, (int)nb2, out);
   return cudaGetLastError();
 }
 

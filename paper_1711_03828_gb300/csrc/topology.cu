@@ -39,6 +39,7 @@
 
 #include "kernels.h"
 #include "draws.cuh"
+#include "square_sum.cuh"
 
 namespace soma {
 
@@ -394,14 +395,15 @@ const void* topology_kernel_ptr(int grid_dtype, bool big, bool types, bool smc) 
              : topology_kernel_ptr_of<false>(grid_dtype, big, types);
 }
 
-// Sum over bonds of |r_i - r_j|^2 (each bond once, from its lower index), FP64.
+// Sum over bonds of |r_i - r_j|^2 (each bond once, from its lower index) and of
+// |r_last - r_0|^2 (square_sum.cuh: exact integers in place of the FP64 pipe).
 __global__ void __launch_bounds__(256) topology_bonds_kernel(
     const Geom g, const float* __restrict__ x, const float* __restrict__ y,
     const float* __restrict__ z, const uint64_t* __restrict__ pmask,
     const uint8_t* __restrict__ mol_arch, const uint8_t* __restrict__ alen,
     double* __restrict__ part) {
   __shared__ double sh[2 * 32];
-  double v = 0.0, re = 0.0;
+  SquareSum bonds, ends;
   const uint64_t M = g.n_chains * g.N;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < M; m += stride) {
@@ -409,52 +411,38 @@ __global__ void __launch_bounds__(256) topology_bonds_kernel(
     const uint32_t i = (uint32_t)(m - mol * g.N);
     const uint32_t a = __ldg(mol_arch + mol);
     const uint64_t pm = __ldg(pmask + a * TOPO_TILE + i);
+    const float x0 = x[m], y0 = y[m], z0 = z[m];
     if (i == 0u) {   // end to end: particle 0 to the architecture's last particle
       const uint64_t e = m + (uint64_t)__ldg(alen + a) - 1u;
-      const double dx = (double)x[e] - (double)x[m];
-      const double dy = (double)y[e] - (double)y[m];
-      const double dz = (double)z[e] - (double)z[m];
-      re += dx * dx + dy * dy + dz * dz;
+      ends.add(x[e], y[e], z[e], x0, y0, z0);
     }
     // partners above i
     for (uint64_t mk = i < 63u ? pm >> (i + 1u) : 0ull; mk; mk &= mk - 1ull) {
       const uint64_t q = m + (uint64_t)__ffsll((long long)mk);
-      const double dx = (double)x[q] - (double)x[m];
-      const double dy = (double)y[q] - (double)y[m];
-      const double dz = (double)z[q] - (double)z[m];
-      v += dx * dx + dy * dy + dz * dz;
+      bonds.add(x[q], y[q], z[q], x0, y0, z0);
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    v += __shfl_xor_sync(FULL, v, o);
-    re += __shfl_xor_sync(FULL, re, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sh[threadIdx.x >> 5] = v;
-    sh[32 + (threadIdx.x >> 5)] = re;
-  }
-  __syncthreads();
+  double v[2] = {bonds.value(), ends.value()};
+  block_sum<2>(v, sh);
   if (threadIdx.x == 0) {
-    double s = 0.0, r = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-      s += sh[k];
-      r += sh[32 + k];
-    }
-    part[2 * blockIdx.x] = s;
-    part[2 * blockIdx.x + 1] = r;
+    part[2 * blockIdx.x] = v[0];
+    part[2 * blockIdx.x + 1] = v[1];
   }
 }
 
-__global__ void topology_bonds_final_kernel(const double* __restrict__ part, int nb,
-                                            double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0, r = 0.0;
-  for (int k = 0; k < nb; ++k) {
-    s += part[2 * k];
-    r += part[2 * k + 1];
+__global__ void __launch_bounds__(256) topology_bonds_final_kernel(const double* __restrict__ part,
+                                                                   int nb, double* __restrict__ out) {
+  __shared__ double sh[2 * 32];
+  double v[2] = {0.0, 0.0};
+  for (int k = threadIdx.x; k < nb; k += 256) {
+    v[0] += part[2 * k];
+    v[1] += part[2 * k + 1];
   }
-  out[0] = s;
-  out[1] = r;
+  block_sum<2>(v, sh);
+  if (threadIdx.x == 0) {
+    out[0] = v[0];
+    out[1] = v[1];
+  }
 }
 
 }  // namespace
@@ -596,7 +584,7 @@ cudaError_t launch_topology_bonds(const Geom& g, const float* x, const float* y,
   uint64_t nb = (M + 255) / 256;
   if (nb > OBS_BLOCKS) nb = OBS_BLOCKS;
   topology_bonds_kernel<<<(unsigned)nb, 256, 0, st>>>(g, x, y, z, pmask, mol_arch, alen, part);
-  topology_bonds_final_kernel<<<1, 32, 0, st>>>(part, (int)nb, out);
+  topology_bonds_final_kernel<<<1, 256, 0, st>>>(part, (int)nb, out);
   return cudaGetLastError();
 }
 

@@ -13,6 +13,7 @@
 // with chi_0ik = chi_ik N / N and every pair of types counted once in the
 // energy (as for two types).
 #include "kernels.h"
+#include "square_sum.cuh"
 
 namespace soma {
 
@@ -133,15 +134,20 @@ __global__ void __launch_bounds__(256) obs_types_kernel(const TypesArgs p, doubl
   }
 }
 
-__global__ void obs_types_final_kernel(const double* __restrict__ part, int nb,
-                                       double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double a = 0.0, b = 0.0;
-  for (int k = 0; k < nb; ++k) {
-    a += part[2 * k];
+__global__ void __launch_bounds__(256) obs_types_final_kernel(const double* __restrict__ part, int nb,
+                                                              double* __restrict__ out) {
+  __shared__ double sh[32], shm[8];
+  double a[1] = {0.0}, b = 0.0;
+  for (int k = threadIdx.x; k < nb; k += 256) {
+    a[0] += part[2 * k];
     b = fmax(b, part[2 * k + 1]);
   }
-  out[2] = a;
+  for (int o = 16; o > 0; o >>= 1) b = fmax(b, __shfl_xor_sync(FULL, b, o));
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = b;
+  block_sum<1>(a, sh);
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) b = fmax(b, shm[k]);
+  out[2] = a[0];
   out[3] = b;
   out[4] = 0.0;
 }
@@ -200,7 +206,7 @@ cudaError_t launch_observables_types(const TypesArgs& a, double kappaN, const ui
   uint64_t nb = ((uint64_t)a.g.cells + 255) / 256;
   if (nb > OBS_BLOCKS) nb = OBS_BLOCKS;
   obs_types_kernel<<<(unsigned)nb, 256, 0, st>>>(a, kappaN, n, part);
-  obs_types_final_kernel<<<1, 32, 0, st>>>(part, (int)nb, out);
+  obs_types_final_kernel<<<1, 256, 0, st>>>(part, (int)nb, out);
   return cudaGetLastError();
 }
 
