@@ -293,14 +293,15 @@ def sweep_kernel_name(d, architectures=False):
         return "sweep_molecule_topology_kernel" if d.set_order == 2 else "sweep_topology_kernel"
     pair = d.N % 2 == 0 and d.N <= 64
     if d.move == 1:
-        return "sweep_smc_pair_kernel" if pair else "sweep_smc_kernel"
+        fills = pair and (64 // d.N) * (d.N // 2 + 1) >= 32   # tiles fill the lanes as strips do
+        return "sweep_smc_pair_kernel" if fills else "sweep_smc_strip_kernel"
     if d.move == 2:
         if not pair or d.flags & 2:
             return "sweep_learned_kernel"
         return "sweep_learned_umma_kernel" if d.flags & 4 else "sweep_learned_tc_kernel"
     if d.set_order == 2:
         return "sweep_molecule_kernel"
-    return "sweep_pair_kernel" if pair else "sweep_uniform_kernel"
+    return "sweep_pair_kernel" if pair else "sweep_strip_kernel"
 
 
 def sweep_kernel_bytes(d, n_types=0):

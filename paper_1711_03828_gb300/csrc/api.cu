@@ -305,7 +305,9 @@ FieldArgs field_args(soma_t* h, int after_sweep) {
   return f;
 }
 
-SweepArgs sweep_args(soma_t* h) {
+// Arguments of the sweep in launch shape sh (the handle's own, or the plain
+// one of the training trajectories).
+SweepArgs sweep_args(soma_t* h, const SweepShape& sh) {
   SweepArgs s;
   s.g = h->g;
   s.x = h->x();
@@ -319,10 +321,13 @@ SweepArgs sweep_args(soma_t* h) {
   s.d_sweep = h->d_counters;
   s.a = h->a32;
   s.K_b = (float)h->K_b;
-  s.G = h->shape.G;
-  s.n_tiles = h->shape.n_tiles;
-  s.full_tiles = h->g.n_chains / h->shape.G;
-  s.last_rows = (uint32_t)(h->g.n_chains % h->shape.G) * h->g.N;
+  s.G = sh.G;
+  s.n_tiles = sh.n_tiles;
+  s.full_tiles = h->g.n_chains / sh.G;
+  s.last_rows = (uint32_t)(h->g.n_chains % sh.G) * h->g.N;
+  s.strip_units = sh.units;
+  s.strip_chains = sh.chains;
+  s.n_items = (uint32_t)sh.n_items;
   s.set_order_random = h->desc.set_order == SOMA_SET_ORDER_RANDOM;
   const double A = h->a64 * h->a64 / 6.0;
   s.smc_A = (float)A;
@@ -433,7 +438,7 @@ cudaError_t launch_sweep_any(soma_t* h, const SweepArgs& sa) {
 }
 
 soma_status one_cycle(soma_t* h) {
-  const SweepArgs sa = sweep_args(h);
+  const SweepArgs sa = sweep_args(h, h->shape);
   soma_status st = timed(h, 0, [&] { return launch_sweep_any(h, sa); });
   if (st != SOMA_OK) return st;
   const FieldArgs fa = field_args(h, 1);
@@ -447,7 +452,7 @@ soma_status one_cycle(soma_t* h) {
 soma_status build_graph(soma_t* h) {
   cudaGraph_t gr = nullptr;
   SOMA_CUDA(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  const SweepArgs sa = sweep_args(h);
+  const SweepArgs sa = sweep_args(h, h->shape);
   const FieldArgs fa = field_args(h, 1);
   const TypesArgs ta = types_args(h, 1);
   cudaError_t e = cudaSuccess;
@@ -577,11 +582,11 @@ soma_status soma_create(const soma_system_desc* desc, soma_t** out) {
   }
 #undef ALLOC
   h->d_out = h->d_scratch + h->scratch_doubles;
-  h->shape = sweep_shape(h->g.n_chains, h->g.N, h->sm_count, h->grid_dtype, desc->move,
+  h->shape = sweep_shape(h->g, h->sm_count, h->grid_dtype, desc->move,
                          (desc->flags & SOMA_FLAG_LEARNED_FP32) != 0,
                          (desc->flags & SOMA_FLAG_LEARNED_UMMA) != 0,
                          desc->set_order == SOMA_ITERATION_MOLECULE);
-  h->plain_shape = sweep_shape(h->g.n_chains, h->g.N, h->sm_count, h->grid_dtype, SOMA_MOVE_UNIFORM);
+  h->plain_shape = sweep_shape(h->g, h->sm_count, h->grid_dtype, SOMA_MOVE_UNIFORM);
 #define CK(call) do { e = (call); if (e != cudaSuccess) { release(h); return cuda_fail(e, #call); } } while (0)
   CK(cudaMemsetAsync(h->n[0], 0, sizeof(uint32_t) * cells, h->stream));
   CK(cudaMemsetAsync(h->n[1], 0, sizeof(uint32_t) * cells, h->stream));
@@ -694,7 +699,7 @@ soma_status soma_shard_sweep(soma_t* h, uint32_t* counts, size_t cells) {
   soma_status st = shard_check(h, counts, cells);
   if (st != SOMA_OK) return st;
   if (h->shard_phase != 0) return fail(SOMA_ESTATE, "soma_shard_fields must come first");
-  const SweepArgs sa = sweep_args(h);
+  const SweepArgs sa = sweep_args(h, h->shape);
   st = timed(h, 0, [&] { return launch_sweep_any(h, sa); });
   if (st != SOMA_OK) return st;
   SOMA_CUDA(cudaMemcpyAsync(counts, h->n[(h->host_sweep + 1) & 1], sizeof(uint32_t) * cells,
@@ -1428,7 +1433,7 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
   SOMA_CUDA(cudaMallocAsync((void**)&dla, sizeof(float) * cfg->batch, h->stream));
   std::vector<float> hJ(cfg->batch), hla(cfg->batch);
   double first = 0.0, last = 0.0, acc_last = 0.0;
-  const SweepArgs sa = sweep_args(h);
+  const SweepArgs sa = sweep_args(h, h->plain_shape);
   const FieldArgs fa = field_args(h, 1);
   for (uint32_t k = 0; k < cfg->steps; ++k) {
     // trajectories of the plain method

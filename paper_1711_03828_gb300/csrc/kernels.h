@@ -14,8 +14,12 @@ struct SweepShape {
   int Q;
   uint32_t G;
   uint64_t n_tiles;
-  bool vec;
   bool pair;  // even N <= 64: one even and one odd particle per lane
+  bool strip;       // the strip layout (strip.cuh), else tiles of whole chains
+  bool wide;        // every axis has two or more cells
+  uint32_t units;   // strips: units per chain, chains per work item, items
+  uint32_t chains;
+  uint64_t n_items;
   bool big;   // 64-bit particle indices (M >= 2^32)
   int move;   // 0 uniform, 1 smart Monte Carlo, 2 learned
   bool learned_tc;  // learned move with the network on the tensor cores
@@ -26,7 +30,7 @@ struct SweepShape {
   int grid;
 };
 
-SweepShape sweep_shape(uint64_t n_chains, uint32_t N, int sm_count, int grid_dtype, int move,
+SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move,
                        bool learned_fp32 = false, bool learned_umma = false,
                        bool molecule = false);
 cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int grid_dtype,
@@ -102,8 +106,8 @@ cudaError_t launch_wait_probe(uint32_t limit, unsigned* err, cudaStream_t st);
 // shared memory (prepare: allow the kernel that much, once at create)
 constexpr int MOL_BLOCK = 128;
 const void* molecule_kernel_ptr(uint32_t N, int grid_dtype, size_t* smem, bool prepare);
-// smart Monte Carlo sweep kernel: paired layout (even N <= 64, 32-bit indices) or general
-const void* smc_kernel_ptr(int Q, bool pair, int grid_dtype);
+// smart Monte Carlo sweep kernel: pair tiles or strips (big: 64-bit indices)
+const void* smc_kernel_ptr(bool strip, bool big);
 // Smart Monte Carlo table (omega and the central-difference field force per
 // type and cell, float4, A then B) from the omega planes of storage type
 // grid_dtype; rebuilt after every field update of a smart Monte Carlo system.

@@ -15,17 +15,11 @@
 // trial position.
 #include "kernels.h"
 #include "pair_body.cuh"
+#include "strip.cuh"
 #include "draws.cuh"
 
 namespace soma {
 
-// ---------------------------------------------------------------------------
-// Smart Monte Carlo (force-biased) step, any N (the tiling of
-// sweep_uniform_kernel).  Trial move dr = A F(r) + sqrt(2A) xi, F = bonded
-// force minus the central-difference gradient of omega_t over the six
-// neighbouring cells; accepted with min(1, exp(-dE) T(r'->r)/T(r->r')),
-// T(r->r') = exp(-|r'-r-A F(r)|^2/(4A)).  Normals and the acceptance uniform
-// from one draw (purpose 1), as above.
 __device__ __forceinline__ void cell3(const Geom& g, float x, float y, float z, uint32_t& cx,
                                       uint32_t& cy, uint32_t& cz) {
   cx = fold_axis(g, 0, x, (uint32_t)g.nx);
@@ -109,160 +103,15 @@ cudaError_t launch_smc_table(const Geom& g, const void* wA, const void* wB, floa
   return cudaGetLastError();
 }
 
-template <int Q>
-__global__ void __launch_bounds__(256) sweep_smc_kernel(const SweepArgs p) {
-  constexpr int S = 2 * Q;
-  const int lane = threadIdx.x & 31;
-  const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const unsigned long long s64 = *p.d_sweep;
-  const uint32_t sweep = (uint32_t)s64;
-  uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
-  const float4* __restrict__ tabA = p.smc_tab;
-  const float4* __restrict__ tabB = p.smc_tab + p.g.cells;
-  const uint32_t N = p.g.N, N_A = p.g.N_A;
-  const uint32_t ctr3a = (PURPOSE_MOVE << 24) | (p.g.replica & 0xFFFFFFu);
-  const uint32_t li0 = (uint32_t)lane * S;
-  const float A = p.smc_A, s2A = p.smc_s2A, inv4A = p.smc_inv4A, K2 = 2.f * p.K_b;
-
-  uint32_t ci[S], src_lane[S], src_slot[S];
-  {
-    uint32_t g = li0 / N, i = li0 - g * N;
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      ci[j] = i;
-      const uint32_t first = g * N;
-      src_lane[j] = (first / S) & 31u;
-      src_slot[j] = first % S;
-      if (++i == N) { i = 0; ++g; }
-    }
-  }
-
-  unsigned my_acc = 0;
-  for (uint64_t tile = warp0; tile < p.n_tiles; tile += nwarps) {
-    const uint64_t chain0 = tile * p.G;
-    const uint64_t rem = p.g.n_chains - chain0;
-    const uint32_t nmono = (rem < p.G ? (uint32_t)rem : p.G) * N;
-    const uint64_t base = chain0 * N + li0;
-
-    float x[S], y[S], z[S];
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      const bool ok = li0 + j < nmono;
-      x[j] = ok ? __ldcs(p.x + base + j) : 0.f;
-      y[j] = ok ? __ldcs(p.y + base + j) : 0.f;
-      z[j] = ok ? __ldcs(p.z + base + j) : 0.f;
-    }
-
-    // configuration-independent part: old cell, field and field force at the
-    // old cell (loaded first, so that the loads are in flight during the
-    // draws), normals, acceptance uniform
-    float gx[S], gy[S], gz[S], lnu[S], w_old[S], fox[S], foy[S], foz[S];
-    uint32_t co[S];
-    uint32_t lowbits = 0;
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      uint32_t cx, cy, cz;
-      cell3(p.g, x[j], y[j], z[j], cx, cy, cz);
-      co[j] = (cz * (uint32_t)p.g.ny + cy) * (uint32_t)p.g.nx + cx;
-      const float4* tab = (ci[j] < N_A) ? tabA : tabB;
-      w_old[j] = 0.f;
-      fox[j] = foy[j] = foz[j] = 0.f;
-      if (li0 + j < nmono) w_old[j] = smc_field(tab, co[j], fox[j], foy[j], foz[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      const uint64_t m = base + j + p.g.id_base;
-      const uint4 r1 = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3a), p.g);
-      lowbits |= (r1.w & 1u) << j;
-      smc_normals(r1, gx[j], gy[j], gz[j]);
-      lnu[j] = log_uniform_open(spare_uniform_word(r1));
-    }
-
-    uint32_t phase[S];
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      uint32_t b = 0;
-      if (p.set_order_random) b = (__shfl_sync(FULL, lowbits, src_lane[j]) >> src_slot[j]) & 1u;
-      phase[j] = (ci[j] & 1u) ^ b;
-    }
-
-#pragma unroll
-    for (uint32_t ph = 0; ph < 2; ++ph) {
-      const float pxl = __shfl_up_sync(FULL, x[S - 1], 1);
-      const float pyl = __shfl_up_sync(FULL, y[S - 1], 1);
-      const float pzl = __shfl_up_sync(FULL, z[S - 1], 1);
-      const float nxl = __shfl_down_sync(FULL, x[0], 1);
-      const float nyl = __shfl_down_sync(FULL, y[0], 1);
-      const float nzl = __shfl_down_sync(FULL, z[0], 1);
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        if (li0 + j >= nmono || phase[j] != ph) continue;
-        const bool hp = ci[j] > 0, hn = ci[j] + 1 < N;
-        const float qx = (j > 0) ? x[j - 1] : pxl, qy = (j > 0) ? y[j - 1] : pyl,
-                    qz = (j > 0) ? z[j - 1] : pzl;
-        const float rx = (j < S - 1) ? x[j + 1] : nxl, ry = (j < S - 1) ? y[j + 1] : nyl,
-                    rz = (j < S - 1) ? z[j + 1] : nzl;
-        // U = sum over bonded partners of (r - n); bonded force = -2 K_b U
-        float ux = 0.f, uy = 0.f, uz = 0.f;
-        if (hp) { ux += x[j] - qx; uy += y[j] - qy; uz += z[j] - qz; }
-        if (hn) { ux += x[j] - rx; uy += y[j] - ry; uz += z[j] - rz; }
-        const float k = (float)((int)hp + (int)hn);
-        const float Fx = fmaf(-K2, ux, fox[j]), Fy = fmaf(-K2, uy, foy[j]), Fz = fmaf(-K2, uz, foz[j]);
-        const float tx = __fadd_rn(x[j], fmaf(s2A, gx[j], A * Fx));
-        const float ty = __fadd_rn(y[j], fmaf(s2A, gy[j], A * Fy));
-        const float tz = __fadd_rn(z[j], fmaf(s2A, gz[j], A * Fz));
-        uint32_t cx, cy, cz;
-        cell3(p.g, tx, ty, tz, cx, cy, cz);
-        const float4* tab = (ci[j] < N_A) ? tabA : tabB;
-        const uint32_t cn = (cz * (uint32_t)p.g.ny + cy) * (uint32_t)p.g.nx + cx;
-        float fnx, fny, fnz;
-        const float w_new = smc_field(tab, cn, fnx, fny, fnz);
-        const float dx = tx - x[j], dy = ty - y[j], dz = tz - z[j];
-        // bonded energy change d.(2U + k d); partners' new U' = U + k d
-        const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
-        const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float dE = fmaf(p.K_b, fmaf(2.f, du, k * dd), w_new - w_old[j]);
-        const float Gx = fmaf(-K2, fmaf(k, dx, ux), fnx), Gy = fmaf(-K2, fmaf(k, dy, uy), fny),
-                    Gz = fmaf(-K2, fmaf(k, dz, uz), fnz);
-        const float ax = dx - A * Fx, ay = dy - A * Fy, az = dz - A * Fz;   // forward residual
-        const float bx = -dx - A * Gx, by = -dy - A * Gy, bz = -dz - A * Gz;  // reverse residual
-        const float fwd = fmaf(ax, ax, fmaf(ay, ay, az * az));
-        const float rev = fmaf(bx, bx, fmaf(by, by, bz * bz));
-        const float log_alpha = fmaf(fwd - rev, inv4A, -dE);
-        if (log_alpha >= 0.f || lnu[j] < log_alpha) {
-          x[j] = tx;
-          y[j] = ty;
-          z[j] = tz;
-          co[j] = cn;
-          ++my_acc;
-        }
-      }
-    }
-
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      if (li0 + j < nmono) {
-        __stcs(p.x + base + j, x[j]);
-        __stcs(p.y + base + j, y[j]);
-        __stcs(p.z + base + j, z[j]);
-        atomicAdd(nacc + co[j], (ci[j] < N_A) ? 1u : 0x10000u);
-      }
-    }
-  }
-
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
-  if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
-}
-
 // ---------------------------------------------------------------------------
 // Smart Monte Carlo step for even N <= 64 in the paired layout of
 // pair_body.cuh: lane l holds the even particle 2l and the odd particle 2l+1
 // of one chain; after the draws the pair is relabelled with the chain's
 // set-order bit into A (moves in the first set) and B (second set), so that
-// every lane moves one particle per set without divergent branches.  The move
-// is the one of sweep_smc_kernel (same draws, same arithmetic per particle).
+// every lane moves one particle per set without divergent branches.  Trial
+// move dr = A F(r) + sqrt(2A) xi, F = bonded force minus the central-difference
+// gradient of omega_t over the six neighbouring cells; accepted with
+// min(1, exp(-dE) T(r'->r)/T(r->r')), T(r->r') = exp(-|r'-r-A F(r)|^2/(4A)).
 struct SmcSlot {
   float x, y, z;      // position
   float gx, gy, gz;   // standard normals
@@ -273,7 +122,7 @@ struct SmcSlot {
 };
 
 __device__ __forceinline__ SmcSlot smc_slot(const Geom& g, const float4* tab, float x, float y, float z,
-                                            uint32_t m, uint32_t sweep, uint32_t ctr3a,
+                                            uint64_t m, uint32_t sweep, uint32_t ctr3a,
                                             bool valid, uint32_t* first_word) {
   SmcSlot q;
   q.x = x; q.y = y; q.z = z;
@@ -284,7 +133,7 @@ __device__ __forceinline__ SmcSlot smc_slot(const Geom& g, const float4* tab, fl
   q.w = 0.f;
   q.fx = q.fy = q.fz = 0.f;
   if (valid) q.w = smc_field(tab, q.c, q.fx, q.fy, q.fz);
-  const uint4 r1 = philox_rk(make_uint4(m, 0u, sweep, ctr3a), g);
+  const uint4 r1 = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3a), g);
   *first_word = r1.w;
   smc_normals(r1, q.gx, q.gy, q.gz);
   q.lnu = log_uniform_open(spare_uniform_word(r1));
@@ -416,10 +265,75 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
   if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
 }
 
-const void* smc_kernel_ptr(int Q, bool pair, int /*grid_dtype: the table is FP32*/) {
-  if (pair) return (const void*)sweep_smc_pair_kernel;
-  return Q == 1 ? (const void*)sweep_smc_kernel<1>
-                : (Q == 2 ? (const void*)sweep_smc_kernel<2> : (const void*)sweep_smc_kernel<4>);
+// Smart Monte Carlo sweep of the other chain lengths, and of even ones whose
+// tiles would leave more slots empty, in the strips of strip.cuh.  2.1M
+// particles of N = 33: 73.9 us a sweep in tiles, 38.5 us in strips.
+template <typename IDX>
+__global__ void __launch_bounds__(768, 1) sweep_smc_strip_kernel(const SweepArgs p) {
+  __shared__ uint32_t s_next;
+  const int lane = threadIdx.x & 31;
+  const uint32_t chunk = (p.n_items + gridDim.x - 1) / gridDim.x;
+  const uint32_t item0 = blockIdx.x * chunk;
+  if (threadIdx.x == 0) s_next = 0u;
+  __syncthreads();
+  const unsigned long long s64 = *p.d_sweep;
+  const uint32_t sweep = (uint32_t)s64;
+  uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
+  const float4* __restrict__ tabA = p.smc_tab;
+  const float4* __restrict__ tabB = p.smc_tab + p.g.cells;
+  const uint32_t N = p.g.N, N_A = p.g.N_A;
+  const uint32_t ctr3 = (PURPOSE_MOVE << 24) | (p.g.replica & 0xFFFFFFu);
+  StripWalk<IDX> walk(p, &s_next, item0, min(item0 + chunk, p.n_items), lane, ctr3, sweep);
+
+  StripPos nv = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float bx = 0.f, by = 0.f, bz = 0.f;   // R of the strip before
+  bool have = walk.step();
+  StripLane<IDX> ns = walk.place();
+  strip_load(p, ns, nv);
+  unsigned my_acc = 0;
+  while (have) {
+    const StripLane<IDX> s = ns;
+    const StripPos v = nv;
+    have = walk.step();
+    ns = walk.place();
+    strip_load(p, ns, nv);
+    const bool aL = s.idx <= N_A, aR = s.idx < N_A;
+    const float4* tL = aL ? tabA : tabB;
+    const float4* tR = aR ? tabA : tabB;
+    uint32_t w;
+    const uint64_t m = (uint64_t)(s.m + (IDX)p.g.id_base);
+    SmcSlot L = smc_slot(p.g, tL, v.Lx, v.Ly, v.Lz, m - 1u, sweep, ctr3, s.vL, &w);
+    SmcSlot R = smc_slot(p.g, tR, v.Rx, v.Ry, v.Rz, m, sweep, ctr3, s.vR, &w);
+    {  // first set: R moves against L of its own and of the next unit
+      const float qx = strip_next(L.x, nv.Lx, lane), qy = strip_next(L.y, nv.Ly, lane),
+                  qz = strip_next(L.z, nv.Lz, lane);
+      const bool a = s.own(), b = s.next(N);
+      my_acc += smc_move(p, tR, R, (a ? R.x - L.x : 0.f) + (b ? R.x - qx : 0.f),
+                         (a ? R.y - L.y : 0.f) + (b ? R.y - qy : 0.f),
+                         (a ? R.z - L.z : 0.f) + (b ? R.z - qz : 0.f), (float)((int)a + (int)b), s.vR);
+    }
+    {  // second set: L moves against R of the previous and of its own unit
+      const float qx = strip_prev(R.x, bx, lane), qy = strip_prev(R.y, by, lane),
+                  qz = strip_prev(R.z, bz, lane);
+      const bool a = s.prev(), b = s.own();
+      my_acc += smc_move(p, tL, L, (a ? L.x - qx : 0.f) + (b ? L.x - R.x : 0.f),
+                         (a ? L.y - qy : 0.f) + (b ? L.y - R.y : 0.f),
+                         (a ? L.z - qz : 0.f) + (b ? L.z - R.z : 0.f), (float)((int)a + (int)b), s.vL);
+    }
+    bx = R.x;
+    by = R.y;
+    bz = R.z;
+    strip_store(p, s, StripPos{L.x, L.y, L.z, R.x, R.y, R.z});
+    strip_count(nacc, s, L.c, R.c, aL ? 1u : 0x10000u, aR ? 1u : 0x10000u);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
+  if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
+}
+
+const void* smc_kernel_ptr(bool strip, bool big) {
+  if (!strip) return (const void*)sweep_smc_pair_kernel;
+  return big ? (const void*)sweep_smc_strip_kernel<uint64_t> : (const void*)sweep_smc_strip_kernel<uint32_t>;
 }
 
 }  // namespace soma

@@ -1,13 +1,12 @@
 // sweep.cu -- the Monte-Carlo step of the SCMF cycle (arXiv:1711.03828,
-// Sec. 2.2 and the SET iteration of Sec. 3.1.2) on sm_103a.
+// Sec. 2.2 and the SET iteration of Sec. 3.1.2) on sm_103a, uniform moves.
 //
-// Work decomposition.  A 32-lane warp owns a tile of G whole chains laid out
-// contiguously (G*N <= 64Q particles).  Lane l holds the 2Q consecutive
-// particles 2Ql .. 2Ql+2Q-1 of the tile in registers, so each lane owns as
-// many even as odd chain positions and BOTH independent sets keep all lanes
-// busy (the paper's SET scheme leaves half its threads idle per set for a
-// linear chain).  Bond partners in a neighbouring lane are exchanged with
-// warp shuffles; no shared memory and no inter-warp synchronisation.
+// Even N <= 64: sweep_pair_kernel (pair_body.cuh), whole chains per warp tile,
+// an even and an odd particle of one chain per lane.  Other lengths:
+// sweep_strip_kernel (strip.cuh), a warp walking along its chains.  Both sets
+// keep all lanes busy (the paper's SET scheme leaves half its threads idle per
+// set for a linear chain); bond partners in a neighbouring lane come by warp
+// shuffles; no shared memory but the counters that hand out the work.
 //
 // Per particle: one Philox4x32-10 draw (counter = particle, sweep) gives the
 // three displacement uniforms and the acceptance uniform; the set order of a
@@ -23,50 +22,39 @@
 // 28 MB grid and the omega planes stay in L2.
 #include "kernels.h"
 #include "pair_body.cuh"
+#include "strip.cuh"
 
 namespace soma {
-
-template <int S>
-__device__ __forceinline__ void load_slots(const float* __restrict__ p, float (&v)[S]) {
-  if constexpr (S == 2) {
-    const float2 t = __ldcs(reinterpret_cast<const float2*>(p));
-    v[0] = t.x;
-    v[1] = t.y;
-  } else {
-#pragma unroll
-    for (int k = 0; k < S / 4; ++k) {
-      const float4 t = __ldcs(reinterpret_cast<const float4*>(p) + k);
-      v[4 * k] = t.x;
-      v[4 * k + 1] = t.y;
-      v[4 * k + 2] = t.z;
-      v[4 * k + 3] = t.w;
-    }
-  }
-}
-
-template <int S>
-__device__ __forceinline__ void store_slots(float* __restrict__ p, const float (&v)[S]) {
-  if constexpr (S == 2) {
-    __stcs(reinterpret_cast<float2*>(p), make_float2(v[0], v[1]));
-  } else {
-#pragma unroll
-    for (int k = 0; k < S / 4; ++k)
-      __stcs(reinterpret_cast<float4*>(p) + k,
-             make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
-  }
-}
 
 __device__ __forceinline__ float dist2(float ax, float ay, float az, float bx, float by, float bz) {
   const float dx = ax - bx, dy = ay - by, dz = az - bz;
   return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
-template <int Q, bool VEC, typename WT>
-__global__ void __launch_bounds__(256) sweep_uniform_kernel(const SweepArgs p) {
-  constexpr int S = 2 * Q;
+// Energy change of the bonds of a particle moved from r to t: partner p (if
+// hp) and q (if hq), each as the difference of the squared lengths.
+__device__ __forceinline__ float bond_change(bool hp, bool hq, float rx, float ry, float rz, float tx,
+                                             float ty, float tz, float px, float py, float pz,
+                                             float qx, float qy, float qz) {
+  const float ep = dist2(tx, ty, tz, px, py, pz) - dist2(rx, ry, rz, px, py, pz);
+  const float eq = dist2(tx, ty, tz, qx, qy, qz) - dist2(rx, ry, rz, qx, qy, qz);
+  return (hp ? ep : 0.f) + (hq ? eq : 0.f);
+}
+
+// Chains of odd length and of more than 64 particles, in the strips of
+// strip.cuh.  One block of 24 warps per SM owns a contiguous range of items,
+// handed out from a shared-memory counter.  WIDE: every axis has two or more
+// cells.  Issue-bound like the paired kernel (454 warp instructions a strip);
+// the paper's thin film (N = 100, 16.5M particles, 16-bit fields): 214 us a
+// sweep in tiles of 128 slots, 152 us in strips.
+template <typename WT, typename IDX, bool WIDE>
+__global__ void __launch_bounds__(768, 1) sweep_strip_kernel(const SweepArgs p) {
+  __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
-  const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint32_t chunk = (p.n_items + gridDim.x - 1) / gridDim.x;
+  const uint32_t item0 = blockIdx.x * chunk;
+  if (threadIdx.x == 0) s_next = 0u;
+  __syncthreads();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
@@ -74,138 +62,104 @@ __global__ void __launch_bounds__(256) sweep_uniform_kernel(const SweepArgs p) {
   const WT* __restrict__ wB = static_cast<const WT*>(p.wB);
   const uint32_t N = p.g.N, N_A = p.g.N_A;
   const uint32_t ctr3 = (PURPOSE_MOVE << 24) | (p.g.replica & 0xFFFFFFu);
-  const uint32_t li0 = (uint32_t)lane * S;
+  StripWalk<IDX> walk(p, &s_next, item0, min(item0 + chunk, p.n_items), lane, ctr3, sweep);
 
-  // Tile-invariant slot metadata: chain-local index, chain within the tile,
-  // and (lane, slot) of that chain's first particle.
-  uint32_t ci[S], src_lane[S], src_slot[S];
-  {
-    uint32_t g = li0 / N, i = li0 - g * N;
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      ci[j] = i;
-      const uint32_t first = g * N;
-      src_lane[j] = (first / S) & 31u;
-      src_slot[j] = first % S;
-      if (++i == N) { i = 0; ++g; }
-    }
-  }
-
+  StripPos nv = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float bx = 0.f, by = 0.f, bz = 0.f;   // R of the strip before
+  bool have = walk.step();
+  StripLane<IDX> ns = walk.place();
+  strip_load(p, ns, nv);
   unsigned my_acc = 0;
-  for (uint64_t tile = warp0; tile < p.n_tiles; tile += nwarps) {
-    const uint64_t chain0 = tile * p.G;
-    const uint64_t rem = p.g.n_chains - chain0;
-    const uint32_t nmono = (rem < p.G ? (uint32_t)rem : p.G) * N;
-    const uint64_t base = chain0 * N + li0;
-    const bool full = li0 + S <= nmono;
+  while (have) {
+    const StripLane<IDX> s = ns;
+    StripPos v = nv;
+    have = walk.step();
+    ns = walk.place();
+    strip_load(p, ns, nv);
 
-    float x[S], y[S], z[S];
-    if (VEC && full) {
-      load_slots<S>(p.x + base, x);
-      load_slots<S>(p.y + base, y);
-      load_slots<S>(p.z + base, z);
-    } else {
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        const bool ok = li0 + j < nmono;
-        x[j] = ok ? __ldcs(p.x + base + j) : 0.f;
-        y[j] = ok ? __ldcs(p.y + base + j) : 0.f;
-        z[j] = ok ? __ldcs(p.z + base + j) : 0.f;
+    // Both slots at once, L low and R high in packed FP32x2 registers: cells,
+    // draws, trial positions as in pair_body.cuh.
+    const unsigned long long MAG = f2_pack(12582912.0f, 12582912.0f);
+    const unsigned long long X = f2_pack(v.Lx, v.Rx), Y = f2_pack(v.Ly, v.Ry), Z = f2_pack(v.Lz, v.Rz);
+    float fx0, fx1, fy0, fy1, fz0, fz1;
+    f2_unpack(f2_add_rm(X, MAG), fx0, fx1);
+    f2_unpack(f2_add_rm(Y, MAG), fy0, fy1);
+    f2_unpack(f2_add_rm(Z, MAG), fz0, fz1);
+    uint32_t cL = cell_of_floor_bits<WIDE>(p.g, __float_as_uint(fx0), __float_as_uint(fy0), __float_as_uint(fz0));
+    uint32_t cR = cell_of_floor_bits<WIDE>(p.g, __float_as_uint(fx1), __float_as_uint(fy1), __float_as_uint(fz1));
+    const bool aL = s.idx <= N_A, aR = s.idx < N_A;   // A particles: idx - 1 < N_A, idx < N_A
+    const WT* __restrict__ wL = aL ? wA : wB;
+    const WT* __restrict__ wR = aR ? wA : wB;
+    // an empty slot's cells lie in the grid too; its values are not used
+    const float oL = load_w<WT>(wL, cL), oR = load_w<WT>(wR, cR);
+    const IDX mR = s.m + (IDX)p.g.id_base, mL = mR - 1u;
+    const uint32_t hL = sizeof(IDX) > 4 ? (uint32_t)((uint64_t)mL >> 32) : 0u;
+    const uint32_t hR = sizeof(IDX) > 4 ? (uint32_t)((uint64_t)mR >> 32) : 0u;
+    const uint4 rL = philox_rk(make_uint4((uint32_t)mL, hL, sweep, ctr3), p.g);
+    const uint4 rR = philox_rk(make_uint4((uint32_t)mR, hR, sweep, ctr3), p.g);
+    const unsigned long long S2 = f2_pack(1.1920928955078125e-7f, 1.1920928955078125e-7f);
+    const unsigned long long C2 = f2_pack(-0.99999994039535522461f, -0.99999994039535522461f);
+    const unsigned long long A2 = f2_pack(p.a, p.a);
+    const unsigned long long XN = f2_fma_rn(
+        A2, f2_fma_rn(f2_pack(__uint2float_rn(rL.x >> 8), __uint2float_rn(rR.x >> 8)), S2, C2), X);
+    const unsigned long long YN = f2_fma_rn(
+        A2, f2_fma_rn(f2_pack(__uint2float_rn(rL.y >> 8), __uint2float_rn(rR.y >> 8)), S2, C2), Y);
+    const unsigned long long ZN = f2_fma_rn(
+        A2, f2_fma_rn(f2_pack(__uint2float_rn(rL.z >> 8), __uint2float_rn(rR.z >> 8)), S2, C2), Z);
+    float txL, txR, tyL, tyR, tzL, tzR;
+    f2_unpack(XN, txL, txR);
+    f2_unpack(YN, tyL, tyR);
+    f2_unpack(ZN, tzL, tzR);
+    f2_unpack(f2_add_rm(XN, MAG), fx0, fx1);
+    f2_unpack(f2_add_rm(YN, MAG), fy0, fy1);
+    f2_unpack(f2_add_rm(ZN, MAG), fz0, fz1);
+    const uint32_t nL = cell_of_floor_bits<WIDE>(p.g, __float_as_uint(fx0), __float_as_uint(fy0), __float_as_uint(fz0));
+    const uint32_t nR = cell_of_floor_bits<WIDE>(p.g, __float_as_uint(fx1), __float_as_uint(fy1), __float_as_uint(fz1));
+    const float dL = load_w<WT>(wL, nL) - oL, dR = load_w<WT>(wR, nR) - oR;
+    float lnuL, lnuR;
+    {
+      float u0, u1;
+      f2_unpack(f2_fma_rn(f2_pack(__uint2float_rn(rL.w >> 8), __uint2float_rn(rR.w >> 8)),
+                          f2_pack(5.9604644775390625e-8f, 5.9604644775390625e-8f),
+                          f2_pack(2.98023223876953125e-8f, 2.98023223876953125e-8f)), u0, u1);
+      lnuL = __logf(u0);
+      lnuR = __logf(u1);
+    }
+
+    {  // first set: R moves
+      const float qx = strip_next(v.Lx, nv.Lx, lane), qy = strip_next(v.Ly, nv.Ly, lane),
+                  qz = strip_next(v.Lz, nv.Lz, lane);
+      const float e = bond_change(s.own(), s.next(N), v.Rx, v.Ry, v.Rz, txR, tyR, tzR, v.Lx, v.Ly,
+                                  v.Lz, qx, qy, qz);
+      const float dE = fmaf(p.K_b, e, dR);
+      if (s.vR && (dE <= 0.f || lnuR < -dE)) {
+        v.Rx = txR;
+        v.Ry = tyR;
+        v.Rz = tzR;
+        cR = nR;
+        ++my_acc;
       }
     }
-
-    // Draws, trial positions, cells and the field change of every slot.
-    float xn[S], yn[S], zn[S], lnu[S], dEf[S];
-    uint32_t co[S], cn[S];
-    uint32_t lowbits = 0;
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      const uint64_t m = base + j + p.g.id_base;
-      const uint4 r = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3), p.g);
-      xn[j] = __fmaf_rn(p.a, uniform_sym(r.x), x[j]);
-      yn[j] = __fmaf_rn(p.a, uniform_sym(r.y), y[j]);
-      zn[j] = __fmaf_rn(p.a, uniform_sym(r.z), z[j]);
-      lnu[j] = log_uniform_open(r.w);
-      lowbits |= (r.w & 1u) << j;
-      co[j] = cell_of(p.g, x[j], y[j], z[j]);
-      cn[j] = cell_of(p.g, xn[j], yn[j], zn[j]);
-      const WT* wt = (ci[j] < N_A) ? wA : wB;
-      dEf[j] = (li0 + j < nmono) ? load_w<WT>(wt, cn[j]) - load_w<WT>(wt, co[j]) : 0.f;
-    }
-
-    // Set of each slot in this sweep: 0 moves first.
-    uint32_t phase[S];
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      uint32_t b = 0;
-      if (p.set_order_random) b = (__shfl_sync(FULL, lowbits, src_lane[j]) >> src_slot[j]) & 1u;
-      phase[j] = (ci[j] & 1u) ^ b;
-    }
-
-#pragma unroll
-    for (uint32_t ph = 0; ph < 2; ++ph) {
-      const float pxl = __shfl_up_sync(FULL, x[S - 1], 1);
-      const float pyl = __shfl_up_sync(FULL, y[S - 1], 1);
-      const float pzl = __shfl_up_sync(FULL, z[S - 1], 1);
-      const float nxl = __shfl_down_sync(FULL, x[0], 1);
-      const float nyl = __shfl_down_sync(FULL, y[0], 1);
-      const float nzl = __shfl_down_sync(FULL, z[0], 1);
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        if (li0 + j >= nmono || phase[j] != ph) continue;
-        const float qx = (j > 0) ? x[j - 1] : pxl;
-        const float qy = (j > 0) ? y[j - 1] : pyl;
-        const float qz = (j > 0) ? z[j - 1] : pzl;
-        const float rx = (j < S - 1) ? x[j + 1] : nxl;
-        const float ry = (j < S - 1) ? y[j + 1] : nyl;
-        const float rz = (j < S - 1) ? z[j + 1] : nzl;
-        float e = 0.f;
-        if (ci[j] > 0)
-          e += dist2(xn[j], yn[j], zn[j], qx, qy, qz) - dist2(x[j], y[j], z[j], qx, qy, qz);
-        if (ci[j] + 1 < N)
-          e += dist2(xn[j], yn[j], zn[j], rx, ry, rz) - dist2(x[j], y[j], z[j], rx, ry, rz);
-        const float dE = fmaf(p.K_b, e, dEf[j]);
-        if (dE <= 0.f || lnu[j] < -dE) {
-          x[j] = xn[j];
-          y[j] = yn[j];
-          z[j] = zn[j];
-          co[j] = cn[j];
-          ++my_acc;
-        }
+    {  // second set: L moves
+      const float px = strip_prev(v.Rx, bx, lane), py = strip_prev(v.Ry, by, lane),
+                  pz = strip_prev(v.Rz, bz, lane);
+      const float e = bond_change(s.prev(), s.own(), v.Lx, v.Ly, v.Lz, txL, tyL, tzL, px, py, pz,
+                                  v.Rx, v.Ry, v.Rz);
+      const float dE = fmaf(p.K_b, e, dL);
+      if (s.vL && (dE <= 0.f || lnuL < -dE)) {
+        v.Lx = txL;
+        v.Ly = tyL;
+        v.Lz = tzL;
+        cL = nL;
+        ++my_acc;
       }
     }
-
-    if (VEC && full) {
-      store_slots<S>(p.x + base, x);
-      store_slots<S>(p.y + base, y);
-      store_slots<S>(p.z + base, z);
-    } else {
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        if (li0 + j < nmono) {
-          __stcs(p.x + base + j, x[j]);
-          __stcs(p.y + base + j, y[j]);
-          __stcs(p.z + base + j, z[j]);
-        }
-      }
-    }
-
-    // Occupation count of the final cells; consecutive slots in one cell are
-    // merged into a single atomic (A adds 1, B adds 1<<16).
-    uint32_t carry = 0;
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      if (li0 + j >= nmono) continue;
-      const uint32_t v = carry + ((ci[j] < N_A) ? 1u : 0x10000u);
-      if (j + 1 < S && li0 + j + 1 < nmono && co[j + 1] == co[j]) {
-        carry = v;
-      } else {
-        atomicAdd(nacc + co[j], v);
-        carry = 0;
-      }
-    }
+    bx = v.Rx;
+    by = v.Ry;
+    bz = v.Rz;
+    strip_store(p, s, v);
+    strip_count(nacc, s, cL, cR, aL ? 1u : 0x10000u, aR ? 1u : 0x10000u);
   }
-
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
   if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
@@ -295,21 +249,20 @@ __global__ void __launch_bounds__(768, 1) sweep_pair_kernel(const SweepArgs p) {
   if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
 }
 
-template <int Q, bool VEC>
-static const void* pick_kernel(int grid_dtype) {
+template <typename IDX, bool WIDE>
+static const void* pick_strip(int grid_dtype) {
   switch (grid_dtype) {
-    case 1: return (const void*)sweep_uniform_kernel<Q, VEC, __nv_bfloat16>;
-    case 2: return (const void*)sweep_uniform_kernel<Q, VEC, __half>;
-    default: return (const void*)sweep_uniform_kernel<Q, VEC, float>;
+    case 1: return (const void*)sweep_strip_kernel<__nv_bfloat16, IDX, WIDE>;
+    case 2: return (const void*)sweep_strip_kernel<__half, IDX, WIDE>;
+    default: return (const void*)sweep_strip_kernel<float, IDX, WIDE>;
   }
 }
 
-static const void* sweep_kernel_ptr(int Q, bool vec, int grid_dtype, bool pair, bool big,
-                                    int move, bool mixed) {
-  if (move == 1) return smc_kernel_ptr(Q, pair && !big, grid_dtype);
-  if (move == 2) return learned_kernel_ptr(Q, grid_dtype);
-  if (pair) {
-    if (big) {
+static const void* sweep_kernel_ptr(const SweepShape& s, int grid_dtype, bool mixed) {
+  if (s.move == 1) return smc_kernel_ptr(s.strip, s.big);
+  if (s.move == 2) return learned_kernel_ptr(s.Q, grid_dtype);
+  if (!s.strip) {
+    if (s.big) {
       switch (grid_dtype) {
         case 1: return (const void*)sweep_pair_kernel<__nv_bfloat16, uint64_t, false>;
         case 2: return (const void*)sweep_pair_kernel<__half, uint64_t, false>;
@@ -329,13 +282,35 @@ static const void* sweep_kernel_ptr(int Q, bool vec, int grid_dtype, bool pair, 
       default: return (const void*)sweep_pair_kernel<float, uint32_t, false>;
     }
   }
-  if (Q == 1) return vec ? pick_kernel<1, true>(grid_dtype) : pick_kernel<1, false>(grid_dtype);
-  if (Q == 2) return vec ? pick_kernel<2, true>(grid_dtype) : pick_kernel<2, false>(grid_dtype);
-  return vec ? pick_kernel<4, true>(grid_dtype) : pick_kernel<4, false>(grid_dtype);
+  if (s.big) return pick_strip<uint64_t, false>(grid_dtype);
+  return s.wide ? pick_strip<uint32_t, true>(grid_dtype) : pick_strip<uint32_t, false>(grid_dtype);
 }
 
-SweepShape sweep_shape(uint64_t n_chains, uint32_t N, int sm_count, int grid_dtype, int move,
-                       bool learned_fp32, bool learned_umma, bool molecule) {
+// Chains per work item of the strip kernels: C chains of U units take
+// ceil(C U / 32) strips (and a draw per chain for the set orders, about a
+// sixth of a strip), n/C items go round `warps` warps.  The C of the lowest
+// time under that count; at most 12 strips (or one chain), so that the warps
+// of a block stay near one another in space.
+static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t warps) {
+  uint32_t best = 1;
+  double least = 0.0;
+  for (uint32_t C = 1; C <= 32u; ++C) {
+    const uint32_t strips = (C * U + 31u) / 32u;
+    if (C > 1u && strips > 12u) break;
+    const uint64_t items = (n + C - 1u) / C;
+    const double cost = (double)((items + warps - 1u) / warps) * ((double)strips + 1.0 / 6.0);
+    if (C == 1u || cost < least) {
+      least = cost;
+      best = C;
+    }
+  }
+  return best;
+}
+
+SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bool learned_fp32,
+                       bool learned_umma, bool molecule) {
+  const uint64_t n_chains = g.n_chains;
+  const uint32_t N = g.N;
   SweepShape s;
   s.move = move;
   s.learned_tc = false;
@@ -345,30 +320,38 @@ SweepShape sweep_shape(uint64_t n_chains, uint32_t N, int sm_count, int grid_dty
   s.Q = (N <= 64) ? 1 : (N <= 128 ? 2 : 4);
   s.G = (uint32_t)(64 * s.Q) / N;
   s.n_tiles = (n_chains + s.G - 1) / s.G;
-  const uint32_t S = 2u * (uint32_t)s.Q;
-  const uint32_t align = S < 4u ? S : 4u;
-  s.vec = ((uint64_t)s.G * N) % align == 0;
   s.pair = (s.Q == 1) && (N % 2 == 0);
   s.big = n_chains * N >= (1ull << 32) || s.n_tiles >= (1ull << 31);
-  // the paired uniform and smart Monte Carlo kernels: one block of 24 warps per SM
-  s.block = ((move == 0 && s.pair) || (move == 1 && s.pair && !s.big)) ? 768 : 256;
-  const void* fn = sweep_kernel_ptr(s.Q, s.vec, grid_dtype, s.pair, s.big, s.move, false);
+  s.wide = g.nx > 1 && g.ny > 1 && g.nz > 1;
+  s.units = N / 2u + 1u;
+  // Uniform moves of even N <= 64 run in pair tiles.  Smart Monte Carlo moves
+  // do where the tiles hold at least as many particles per slot as the strips
+  // (G N of 64 slots against N of 2 U) and the indices fit 32 bits.
+  s.strip = !s.pair || (move == 1 && (s.big || s.G * s.units < 32u));
+  if (move == 2 || (molecule && move == 0)) s.strip = false;
+  s.block = 256;
   if (move == 2 && s.pair && !s.big && !learned_fp32) {
     s.learned_tc = true;
     s.learned_umma = learned_umma;
     s.block = 128;
-    fn = learned_tc_kernel_ptr(grid_dtype, s.learned_umma);
-  }
-  if (molecule && move == 0) {
+  } else if (molecule && move == 0) {
     s.molecule = true;
     s.block = MOL_BLOCK;
-    fn = molecule_kernel_ptr(N, grid_dtype, &s.smem, true);
+  } else if (move != 2) {
+    s.block = 768;   // one block of 24 warps per SM
   }
+  s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
+  s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
+  const void* fn = s.learned_tc ? learned_tc_kernel_ptr(grid_dtype, s.learned_umma)
+                 : s.molecule   ? molecule_kernel_ptr(N, grid_dtype, &s.smem, true)
+                                : sweep_kernel_ptr(s, grid_dtype, false);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, s.smem);
   if (per_sm < 1) per_sm = 1;
   const uint64_t warps_per_block = (uint64_t)s.block / 32;
+  // a strip launch spreads its items over all SMs, however few they are
   const uint64_t need = s.molecule ? (n_chains + s.block - 1) / s.block
+                      : s.strip    ? s.n_items
                                    : (s.n_tiles + warps_per_block - 1) / warps_per_block;
   const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
   s.grid = (int)(need < cap ? need : cap);
@@ -380,8 +363,7 @@ cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int gr
                                  cudaStream_t st) {
   size_t smem = 0;
   const void* fn = s.molecule ? molecule_kernel_ptr(a.g.N, grid_dtype, &smem, false)
-                              : sweep_kernel_ptr(s.Q, s.vec, grid_dtype, s.pair, s.big, s.move,
-                                                 a.seq != nullptr);
+                              : sweep_kernel_ptr(s, grid_dtype, a.seq != nullptr);
   void* args[] = {const_cast<SweepArgs*>(&a)};
   return cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st);
 }
