@@ -118,6 +118,8 @@ struct soma_t {
   uint32_t* nt[2] = {nullptr, nullptr};      // count planes, n_types * cells each
   float* wt = nullptr;                       // field planes, n_types * cells
   int topo_grid = 1;
+  uint4* d_topo_pair = nullptr;              // 256 * 32 set pairs (topology_pairs)
+  uint32_t topo_R = 0, topo_G = 0;           // lanes, molecules per tile (0: general kernel)
   double* d_out = nullptr;
   size_t scratch_doubles = 0;
   double* d_tw = nullptr;                    // S(q): twiddles of the axes, results (lazy)
@@ -273,6 +275,7 @@ void release(soma_t* h) {
   cudaFree(h->d_topo_ptab);
   cudaFree(h->d_topo_ttab);
   cudaFree(h->d_topo_len);
+  cudaFree(h->d_topo_pair);
   cudaFree(h->nt[0]);
   cudaFree(h->nt[1]);
   cudaFree(h->wt);
@@ -383,6 +386,9 @@ TopoArgs topo_args(soma_t* h, const SweepArgs& sa) {
   t.wt = h->wt;
   t.nt0 = h->nt[0];
   t.nt1 = h->nt[1];
+  t.pair_tab = h->d_topo_pair;
+  t.pair_R = h->topo_R;
+  t.pair_G = h->topo_G;
   return t;
 }
 
@@ -429,6 +435,9 @@ cudaError_t launch_sweep_any(soma_t* h, const SweepArgs& sa) {
   if (h->has_topo && h->shape.molecule)
     return launch_molecule_topology(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->stream,
                                     types);
+  if (h->has_topo && h->topo_R)
+    return launch_sweep_topology_pair(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->stream, types,
+                                      h->desc.move == SOMA_MOVE_SMC);
   if (h->has_topo)
     return launch_sweep_topology(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->shape.big,
                                  h->stream, types, h->desc.move == SOMA_MOVE_SMC);
@@ -927,6 +936,7 @@ namespace {
 void set_topo_grid(soma_t* h) {
   h->topo_grid = h->shape.molecule
                      ? molecule_topology_grid(h->g.N, h->grid_dtype, h->sm_count, h->g.n_chains)
+                 : h->topo_R ? topology_pair_grid(h->g.n_chains, h->topo_G, h->sm_count)
                      : topology_grid(h->grid_dtype, h->shape.big, h->sm_count, h->shape.n_tiles,
                                      h->n_types != 0, h->desc.move == SOMA_MOVE_SMC);
 }
@@ -969,6 +979,7 @@ soma_status soma_set_topology(soma_t* h, const uint32_t* words, uint64_t n_words
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_topo_ptab, sizeof(uint32_t) * 256 * 64);
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_topo_ttab, 256 * 64);
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_topo_len, 256);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_topo_pair, sizeof(uint4) * 256 * 32);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc architecture tables");
   }
   if (!h->d_seq) {
@@ -986,6 +997,10 @@ soma_status soma_set_topology(soma_t* h, const uint32_t* words, uint64_t n_words
                             h->stream));
   SOMA_CUDA(cudaMemcpyAsync(h->d_topo_ttab, T.ttab.data(), T.ttab.size(), up, h->stream));
   SOMA_CUDA(cudaMemcpyAsync(h->d_topo_len, T.len.data(), T.len.size(), up, h->stream));
+  const TopologyPairs pairs = h->shape.big ? TopologyPairs() : topology_pairs(T, n_arch, h->g.N);
+  if (pairs.R)
+    SOMA_CUDA(cudaMemcpyAsync(h->d_topo_pair, pairs.tab.data(), sizeof(uint4) * pairs.tab.size(), up,
+                              h->stream));
   SOMA_CUDA(cudaMemcpyAsync(h->d_seq, T.seq.data(), sizeof(uint64_t) * n_arch, up, h->stream));
   SOMA_CUDA(cudaMemcpyAsync(h->d_arch, a.data(), a.size(), up, h->stream));
   soma_status s2 = sync(h);   // the host vectors are released on return
@@ -999,6 +1014,8 @@ soma_status soma_set_topology(soma_t* h, const uint32_t* words, uint64_t n_words
     h->g.particles = present;
     h->rho_cell = (double)present / (double)h->g.cells;
   }
+  h->topo_R = pairs.R;
+  h->topo_G = pairs.G;
   h->has_topo = true;
   set_topo_grid(h);
   if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }

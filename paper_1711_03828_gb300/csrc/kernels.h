@@ -135,6 +135,11 @@ struct TopoArgs {
   const float* wt;
   uint32_t* nt0;
   uint32_t* nt1;
+  // architectures of at most two sets: [a*32 + rank] = table words of the
+  // rank-th particles of set 0 and set 1, and particle0 | particle1 << 8 |
+  // type0 << 16 | type1 << 24 (0xFF: none); lanes and molecules per warp tile
+  const uint4* pair_tab;
+  uint32_t pair_R, pair_G;
 };
 struct TopologyTables {
   std::vector<uint64_t> pmask;   // n_arch * 64
@@ -154,6 +159,17 @@ struct TopologyTables {
 std::string topology_tables(const uint32_t* words, uint64_t n_words, const uint32_t* start,
                             uint32_t n_arch, uint32_t N, TopologyTables* out,
                             uint32_t n_types = 2);
+// Pairs of one particle of set 0 and one of set 1 per lane; R = 0 where some
+// architecture has more than two sets or a warp would hold fewer molecules than
+// a tile of the general kernel.
+struct TopologyPairs {
+  std::vector<uint4> tab;
+  uint32_t R = 0, G = 0;
+};
+TopologyPairs topology_pairs(const TopologyTables& T, uint32_t n_arch, uint32_t N);
+int topology_pair_grid(uint64_t n_mol, uint32_t G, int sm_count);
+cudaError_t launch_sweep_topology_pair(const TopoArgs& a, int grid, int grid_dtype, cudaStream_t st,
+                                       bool types, bool smc);
 // smc: the smart Monte Carlo move (the table s.smc_tab holds one plane per type)
 int topology_grid(int grid_dtype, bool big, int sm_count, uint64_t n_tiles, bool types = false,
                   bool smc = false);

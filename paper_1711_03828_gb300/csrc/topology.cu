@@ -93,6 +93,7 @@ __device__ __forceinline__ uint32_t pw_partner(uint32_t w, int k) { return (w >>
 __device__ __forceinline__ bool pw_is_B(uint32_t w) { return (w >> 24) & 1u; }
 __device__ __forceinline__ uint32_t pw_set(uint32_t w) { return (w >> 25) & 7u; }
 __device__ __forceinline__ uint32_t pw_sets(uint32_t w) { return w >> 28; }
+inline uint32_t pw_set_of(uint32_t w) { return (w >> 25) & 7u; }   // host
 
 // Shared-memory record of one warp's tile, one 16-byte entry per particle and
 // array (a mover reads each with one 128-bit access), entry q at slot
@@ -369,6 +370,264 @@ __global__ void __launch_bounds__(256, 3) sweep_topology_kernel(const TopoArgs t
   if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
 }
 
+// Architectures of one or two sets (trees, even rings): each lane owns one
+// particle of set 0 and one of set 1 of the same molecule, paired by their rank
+// in the set (pair_tab), so that a step moves one particle of every lane
+// without mover lists and a particle's draw, trial position, cells, field
+// change and table word stay in its lane's registers.  Only the current
+// positions go to shared memory, where a mover reads its bond partners.  A warp
+// owns G molecules, R lanes each (R: the largest set of any architecture); one
+// block of 24 warps per SM takes its tiles from a shared-memory counter; the
+// next tile's positions and the architectures of the one after are loaded
+// ahead.  The moves are those of sweep_topology_kernel, operation for operation.
+// Stars, combs, rings and diblocks of 32 (16.8M particles): 252 us a sweep with
+// mover lists (695 warp instructions a tile), 196 us in pairs (609); three types
+// under smart Monte Carlo (2.1M): 47.0 and 44.9 us.
+struct TopoSlot {
+  float x, y, z, tx, ty, tz;   // position, trial (smart Monte Carlo: normals)
+  float thr;                   // acceptance threshold (smart Monte Carlo: ln u)
+  float w, fx, fy, fz;         // smart Monte Carlo: omega and field force at the old cell
+  uint32_t c, cn;              // old cell, trial cell
+  uint32_t pw, i, type;        // table word, particle of the molecule, type
+  bool valid;
+};
+
+template <typename WT, bool MULTI, bool SMC>
+__device__ __forceinline__ void topo_draw(const TopoArgs& t, TopoSlot& s, const uint4& r) {
+  const SweepArgs& p = t.s;
+  if (SMC) {
+    smc_normals(r, s.tx, s.ty, s.tz);
+    s.thr = log_uniform_open(spare_uniform_word(r));
+  } else {
+    s.tx = __fmaf_rn(p.a, uniform_sym(r.x), s.x);
+    s.ty = __fmaf_rn(p.a, uniform_sym(r.y), s.y);
+    s.tz = __fmaf_rn(p.a, uniform_sym(r.z), s.z);
+    s.cn = cell_of(p.g, s.tx, s.ty, s.tz);
+    float dEf;
+    if (MULTI) {
+      const float* wt = t.wt + (size_t)s.type * p.g.cells;
+      dEf = __ldg(wt + s.cn) - __ldg(wt + s.c);
+    } else {
+      const WT* wt = static_cast<const WT*>(s.type ? p.wB : p.wA);
+      dEf = load_w<WT>(wt, s.cn) - load_w<WT>(wt, s.c);
+    }
+    s.thr = -log_uniform_open(r.w) - dEf;
+  }
+}
+
+// Moves s against the positions P of its molecule's particles; returns
+// acceptance (s then holds the new position and cell).
+template <bool SMC>
+__device__ __forceinline__ bool topo_move(const TopoArgs& t, TopoSlot& s, const float4* P,
+                                          uint32_t mol0, uint32_t arch) {
+  const SweepArgs& p = t.s;
+  const uint32_t deg = pw_degree(s.pw);
+  float ux = 0.f, uy = 0.f, uz = 0.f;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    if ((uint32_t)b < deg) {
+      const float4 n = P[TopoTile<false>::rec(mol0 + pw_partner(s.pw, b))];
+      ux += s.x - n.x;
+      uy += s.y - n.y;
+      uz += s.z - n.z;
+    }
+  }
+  if (deg > 3u) {   // the partners after the third, from the full mask
+    uint64_t mk = __ldg(t.pmask + arch * TOPO_TILE + s.i);
+    mk &= mk - 1ull;
+    mk &= mk - 1ull;
+    mk &= mk - 1ull;
+    for (; mk; mk &= mk - 1ull) {
+      const float4 n = P[TopoTile<false>::rec(mol0 + (uint32_t)__ffsll((long long)mk) - 1u)];
+      ux += s.x - n.x;
+      uy += s.y - n.y;
+      uz += s.z - n.z;
+    }
+  }
+  if (SMC) {
+    const float4* __restrict__ tab = p.smc_tab + (size_t)s.type * p.g.cells;
+    const float A = p.smc_A, K2 = 2.f * p.K_b, k = (float)deg;
+    float fnx, fny, fnz;
+    const float Fx = fmaf(-K2, ux, s.fx), Fy = fmaf(-K2, uy, s.fy), Fz = fmaf(-K2, uz, s.fz);
+    const float tx = __fadd_rn(s.x, fmaf(p.smc_s2A, s.tx, A * Fx));
+    const float ty = __fadd_rn(s.y, fmaf(p.smc_s2A, s.ty, A * Fy));
+    const float tz = __fadd_rn(s.z, fmaf(p.smc_s2A, s.tz, A * Fz));
+    const uint32_t cn = cell_of(p.g, tx, ty, tz);
+    const float w_new = smc_field(tab, cn, fnx, fny, fnz);
+    const float dx = tx - s.x, dy = ty - s.y, dz = tz - s.z;
+    // bonded energy change d.(2U + k d); the force at r' uses U' = U + k d
+    const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
+    const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float dE = fmaf(p.K_b, fmaf(2.f, du, k * dd), w_new - s.w);
+    const float Gx = fmaf(-K2, fmaf(k, dx, ux), fnx), Gy = fmaf(-K2, fmaf(k, dy, uy), fny),
+                Gz = fmaf(-K2, fmaf(k, dz, uz), fnz);
+    const float ax = dx - A * Fx, ay = dy - A * Fy, az = dz - A * Fz;     // forward residual
+    const float bx = -dx - A * Gx, by = -dy - A * Gy, bz = -dz - A * Gz;  // reverse residual
+    const float fwd = fmaf(ax, ax, fmaf(ay, ay, az * az));
+    const float rev = fmaf(bx, bx, fmaf(by, by, bz * bz));
+    const float log_alpha = fmaf(fwd - rev, p.smc_inv4A, -dE);
+    const bool acc = s.valid && (log_alpha >= 0.f || s.thr < log_alpha);
+    s.x = acc ? tx : s.x;
+    s.y = acc ? ty : s.y;
+    s.z = acc ? tz : s.z;
+    s.c = acc ? cn : s.c;
+    return acc;
+  } else {
+    const float dx = s.tx - s.x, dy = s.ty - s.y, dz = s.tz - s.z;
+    const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
+    const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const bool acc = s.valid && p.K_b * fmaf(2.f, du, (float)deg * dd) <= s.thr;
+    s.x = acc ? s.tx : s.x;
+    s.y = acc ? s.ty : s.y;
+    s.z = acc ? s.tz : s.z;
+    s.c = acc ? s.cn : s.c;
+    return acc;
+  }
+}
+
+template <typename WT, bool MULTI, bool SMC>
+__global__ void __launch_bounds__(768, 1) sweep_topology_pair_kernel(const TopoArgs t) {
+  __shared__ uint32_t s_next;
+  __shared__ float4 record[24][TopoTile<false>::REC];
+  const SweepArgs& p = t.s;
+  const int lane = threadIdx.x & 31;
+  float4* P = record[threadIdx.x >> 5];
+  const uint32_t n_mol = (uint32_t)p.g.n_chains, N = p.g.N, G = t.pair_G, R = t.pair_R;
+  const uint32_t n_tiles = (n_mol + G - 1u) / G;
+  const uint32_t chunk = (n_tiles + gridDim.x - 1) / gridDim.x;
+  const uint32_t t_begin = blockIdx.x * chunk;
+  const uint32_t t_end = min(t_begin + chunk, n_tiles);
+  if (threadIdx.x == 0) s_next = 0u;
+  __syncthreads();
+  auto claim = [&]() -> uint32_t {
+    uint32_t v = 0u;
+    if (lane == 0) v = atomicAdd(&s_next, 1u);
+    return t_begin + __shfl_sync(FULL, v, 0);
+  };
+  const unsigned long long s64 = *p.d_sweep;
+  const uint32_t sweep = (uint32_t)s64;
+  uint32_t* __restrict__ nacc = MULTI ? (((s64 + 1ull) & 1ull) ? t.nt1 : t.nt0)
+                                      : (((s64 + 1ull) & 1ull) ? p.n1 : p.n0);
+  const uint32_t ctr3 = (PURPOSE_MOVE << 24) | (p.g.replica & 0xFFFFFFu);
+  const bool random = p.set_order_random != 0;
+  const uint32_t g = (uint32_t)lane / R, rank = (uint32_t)lane - g * R;
+  const bool lane_in = g < G;
+  const uint32_t mol0 = g * N;                   // tile index of the molecule's particle 0
+
+  // architecture of this lane's molecule in a tile (0 where there is none)
+  auto load_arch = [&](uint32_t tile) -> uint32_t {
+    const uint32_t m = tile * G + g;
+    return (tile < t_end && lane_in && m < n_mol) ? (uint32_t)__ldg(t.mol_arch + m) : 0u;
+  };
+  // table entry and positions of this lane's two particles in a tile
+  uint4 e;                                       // table words 0, 1; particles and types
+  float px0 = 0.f, py0 = 0.f, pz0 = 0.f, px1 = 0.f, py1 = 0.f, pz1 = 0.f;
+  auto load_tile = [&](uint32_t tile, uint32_t a) {
+    const uint32_t m = tile * G + g;
+    e = make_uint4(0u, 0u, 0xFFFFu, 0u);
+    if (tile < t_end && lane_in && m < n_mol) {
+      e = __ldg(t.pair_tab + a * 32u + rank);
+      const uint32_t b = m * N, i0 = e.z & 0xFFu, i1 = (e.z >> 8) & 0xFFu;
+      if (i0 != 0xFFu) {
+        px0 = __ldcs(p.x + (b + i0));
+        py0 = __ldcs(p.y + (b + i0));
+        pz0 = __ldcs(p.z + (b + i0));
+      }
+      if (i1 != 0xFFu) {
+        px1 = __ldcs(p.x + (b + i1));
+        py1 = __ldcs(p.y + (b + i1));
+        pz1 = __ldcs(p.z + (b + i1));
+      }
+    }
+  };
+  uint32_t tile = claim();
+  uint32_t arch = load_arch(tile);
+  load_tile(tile, arch);
+  uint32_t tile1 = claim();
+  uint32_t arch1 = load_arch(tile1);
+
+  unsigned my_acc = 0;
+  while (tile < t_end) {
+    TopoSlot a, b;
+    a.x = px0; a.y = py0; a.z = pz0;
+    b.x = px1; b.y = py1; b.z = pz1;
+    a.pw = e.x;
+    b.pw = e.y;
+    a.i = e.z & 0xFFu;
+    b.i = (e.z >> 8) & 0xFFu;
+    a.type = (e.z >> 16) & 0xFFu;
+    b.type = e.z >> 24;
+    a.valid = a.i != 0xFFu;
+    b.valid = b.i != 0xFFu;
+    const uint32_t m0 = (tile * G + g) * N, this_arch = arch;
+    // the next tile's positions, and the architectures of the one after
+    load_tile(tile1, arch1);
+    tile = tile1;
+    arch = arch1;
+    tile1 = claim();
+    arch1 = load_arch(tile1);
+
+    if (a.valid) P[TopoTile<false>::rec(mol0 + a.i)] = make_float4(a.x, a.y, a.z, 0.f);
+    if (b.valid) P[TopoTile<false>::rec(mol0 + b.i)] = make_float4(b.x, b.y, b.z, 0.f);
+    a.c = cell_of(p.g, a.x, a.y, a.z);
+    b.c = cell_of(p.g, b.x, b.y, b.z);
+    if (SMC) {   // an empty slot's cell lies in the grid; its values are not used
+      a.w = smc_field(p.smc_tab + (size_t)a.type * p.g.cells, a.c, a.fx, a.fy, a.fz);
+      b.w = smc_field(p.smc_tab + (size_t)b.type * p.g.cells, b.c, b.fx, b.fy, b.fz);
+    }
+    const uint32_t id0 = m0 + a.i + (uint32_t)p.g.id_base, id1 = m0 + b.i + (uint32_t)p.g.id_base;
+    const uint4 r0 = philox_rk(make_uint4(id0, 0u, sweep, ctr3), p.g);
+    const uint4 r1 = philox_rk(make_uint4(id1, 0u, sweep, ctr3), p.g);
+    topo_draw<WT, MULTI, SMC>(t, a, r0);
+    topo_draw<WT, MULTI, SMC>(t, b, r1);
+    // particle 0 is the first of set 0: its acceptance word orders the sets
+    const bool sw = random && (__shfl_sync(FULL, r0.w, (int)(g * R) & 31) & 1u);
+    TopoSlot A = sw ? b : a, B = sw ? a : b;   // A moves first
+    __syncwarp();
+    my_acc += topo_move<SMC>(t, A, P, mol0, this_arch);
+    __syncwarp();   // every mover has read its partners (none of its own set)
+    if (A.valid) P[TopoTile<false>::rec(mol0 + A.i)] = make_float4(A.x, A.y, A.z, 0.f);
+    __syncwarp();
+    my_acc += topo_move<SMC>(t, B, P, mol0, this_arch);
+    __syncwarp();   // before the next tile's positions replace these
+
+    if (A.valid) {
+      __stcs(p.x + (m0 + A.i), A.x);
+      __stcs(p.y + (m0 + A.i), A.y);
+      __stcs(p.z + (m0 + A.i), A.z);
+    }
+    if (B.valid) {
+      __stcs(p.x + (m0 + B.i), B.x);
+      __stcs(p.y + (m0 + B.i), B.y);
+      __stcs(p.z + (m0 + B.i), B.z);
+    }
+    if (MULTI) {
+      const bool same = A.valid && B.valid && A.c == B.c && A.type == B.type;
+      if (A.valid) atomicAdd(nacc + (size_t)A.type * p.g.cells + A.c, same ? 2u : 1u);
+      if (B.valid && !same) atomicAdd(nacc + (size_t)B.type * p.g.cells + B.c, 1u);
+    } else {
+      const uint32_t vA = A.type ? 0x10000u : 1u, vB = B.type ? 0x10000u : 1u;
+      const bool same = A.valid && B.valid && A.c == B.c;
+      if (A.valid) atomicAdd(nacc + A.c, same ? vA + vB : vA);
+      if (B.valid && !same) atomicAdd(nacc + B.c, vB);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
+  if (lane == 0 && my_acc) atomicAdd(p.acc, (unsigned long long)my_acc);
+}
+
+template <bool SMC>
+const void* topology_pair_ptr_of(int grid_dtype, bool types) {
+  if (types) return (const void*)sweep_topology_pair_kernel<float, true, SMC>;   // FP32 fields only
+  if (SMC) return (const void*)sweep_topology_pair_kernel<float, false, SMC>;    // FP32 table
+  switch (grid_dtype) {
+    case 1: return (const void*)sweep_topology_pair_kernel<__nv_bfloat16, false, false>;
+    case 2: return (const void*)sweep_topology_pair_kernel<__half, false, false>;
+    default: return (const void*)sweep_topology_pair_kernel<float, false, false>;
+  }
+}
+
 template <bool SMC>
 const void* topology_kernel_ptr_of(int grid_dtype, bool big, bool types) {
   // the smart Monte Carlo move reads the FP32 table, whatever the field storage
@@ -556,6 +815,55 @@ std::string topology_tables(const uint32_t* w, uint64_t n_words, const uint32_t*
     }
   }
   return std::string();
+}
+
+TopologyPairs topology_pairs(const TopologyTables& T, uint32_t n_arch, uint32_t N) {
+  TopologyPairs P;
+  uint32_t R = 1;
+  for (uint32_t a = 0; a < n_arch; ++a) {
+    if (T.nsets[a] > 2u) return P;
+    uint32_t cnt[2] = {0, 0};
+    for (uint32_t i = 0; i < T.len[a]; ++i) ++cnt[pw_set_of(T.ptab[(size_t)a * TOPO_TILE + i])];
+    R = std::max(R, std::max(cnt[0], cnt[1]));
+  }
+  if (R > 32u) return P;
+  // only where a warp then holds as many molecules as a tile of the general
+  // kernel, floor(64/N): pairs take 0.78 (uniform) to 0.95 (smart Monte Carlo)
+  // of its time for the same molecules, which a smaller tile would use up
+  const uint32_t G = std::min(32u / R, (uint32_t)TOPO_TILE / N);
+  if (G < (uint32_t)TOPO_TILE / N) return P;
+  P.tab.assign((size_t)n_arch * 32, make_uint4(0u, 0u, 0xFFFFu, 0u));
+  for (uint32_t a = 0; a < n_arch; ++a) {
+    uint32_t at[2] = {0, 0};
+    for (uint32_t i = 0; i < T.len[a]; ++i) {
+      const uint32_t w = T.ptab[(size_t)a * TOPO_TILE + i], s = pw_set_of(w);
+      const uint32_t type = T.ttab[(size_t)a * TOPO_TILE + i];
+      uint4& e = P.tab[(size_t)a * 32 + at[s]++];
+      if (s == 0u) {
+        e.x = w;
+        e.z = (e.z & 0xFF00FF00u) | i | type << 16;
+      } else {
+        e.y = w;
+        e.z = (e.z & 0x00FF00FFu) | i << 8 | type << 24;
+      }
+    }
+  }
+  P.R = R;
+  P.G = G;
+  return P;
+}
+
+int topology_pair_grid(uint64_t n_mol, uint32_t G, int sm_count) {
+  const uint64_t tiles = (n_mol + G - 1u) / G;   // spread over all SMs, however few
+  return (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)sm_count));
+}
+
+cudaError_t launch_sweep_topology_pair(const TopoArgs& a, int grid, int grid_dtype, cudaStream_t st,
+                                       bool types, bool smc) {
+  void* args[] = {const_cast<TopoArgs*>(&a)};
+  return cudaLaunchKernel(smc ? topology_pair_ptr_of<true>(grid_dtype, types)
+                              : topology_pair_ptr_of<false>(grid_dtype, types),
+                          dim3(grid), dim3(768), args, 0, st);
 }
 
 int topology_grid(int grid_dtype, bool big, int sm_count, uint64_t n_tiles, bool types, bool smc) {
