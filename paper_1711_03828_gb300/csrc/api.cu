@@ -788,20 +788,40 @@ soma_status soma_get_positions(soma_t* h, float* dst, size_t n, int dst_on_devic
   return sync(h);
 }
 
+namespace {
+// Device memory of the current device (a kernel may read it); managed memory,
+// another device's and anything unknown go through a copy call.
+bool on_this_device(const void* p) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+}  // namespace
+
 soma_status soma_set_positions(soma_t* h, const float* src, size_t n, int src_on_device) {
   if (!h || !src) return fail(SOMA_EINVAL, "NULL argument");
   if (n != 3 * h->M) return fail(SOMA_EINVAL, "n=%zu, expected 3*M=%llu", n, (unsigned long long)(3 * h->M));
-  const cudaMemcpyKind k = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  for (int d = 0; d < 3; ++d)
-    SOMA_CUDA(cudaMemcpyAsync(h->pos + d * h->plane, src + d * h->M, sizeof(float) * h->M, k, h->stream));
   // every coordinate must lie in the supported range of the cell fold; the
   // check runs on the device copy, and a handle holding positions outside it
   // refuses to sweep until valid positions are set
   const float lim = (float)POS_LIMIT;
   unsigned flag = 0;
   SOMA_CUDA(cudaMemsetAsync(h->d_err + 2, 0, sizeof(unsigned), h->stream));
-  for (int d = 0; d < 3; ++d)
-    SOMA_CUDA(launch_range_check(h->pos + d * h->plane, h->M, lim, h->d_err + 2, h->sm_count, h->stream));
+  if (src_on_device && on_this_device(src)) {
+    SOMA_CUDA(launch_copy_check(src, h->pos, h->M, h->plane, lim, h->d_err + 2, h->sm_count, h->stream));
+  } else {
+    const cudaMemcpyKind k = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    for (int d = 0; d < 3; ++d) {
+      SOMA_CUDA(cudaMemcpyAsync(h->pos + d * h->plane, src + d * h->M, sizeof(float) * h->M, k,
+                                h->stream));
+      SOMA_CUDA(launch_range_check(h->pos + d * h->plane, h->M, lim, h->d_err + 2, h->sm_count,
+                                   h->stream));
+    }
+  }
   SOMA_CUDA(cudaMemcpyAsync(&flag, h->d_err + 2, sizeof flag, cudaMemcpyDeviceToHost, h->stream));
   SOMA_CUDA(cudaStreamSynchronize(h->stream));
   h->launches += 3;

@@ -50,6 +50,9 @@ cudaError_t launch_histogram(const Geom& g, const float* x, const float* y, cons
                              uint32_t* n, int sm_count, cudaStream_t st,
                              const uint64_t* seq = nullptr, const uint8_t* arch = nullptr,
                              const uint8_t* alen = nullptr);
+// the same for positions on this device, copied on the way: dst + d plane = src + d n, d < 3
+cudaError_t launch_copy_check(const float* src, float* dst, uint64_t n, uint64_t plane, float lim,
+                              unsigned* flag, int sm_count, cudaStream_t st);
 cudaError_t launch_range_check(const float* p, uint64_t n, float lim, unsigned* flag, int sm_count,
                                cudaStream_t st);
 cudaError_t launch_fields(const FieldArgs& a, unsigned* arrive, int grid_dtype, int sm_count,
