@@ -478,17 +478,15 @@ soma_status build_graph(soma_t* h) {
   return SOMA_OK;
 }
 
-soma_status check_sticky(soma_t* h) {
+// Waits for the stream with one copy of the sticky error word behind its work
+// (a wait and then a blocking copy waited twice).
+soma_status sync(soma_t* h) {
   unsigned err = 0;
-  SOMA_CUDA(cudaMemcpy(&err, h->d_err, sizeof err, cudaMemcpyDeviceToHost));
+  SOMA_CUDA(cudaMemcpyAsync(&err, h->d_err, sizeof err, cudaMemcpyDeviceToHost, h->stream));
+  SOMA_CUDA(cudaStreamSynchronize(h->stream));
   if (err & ERR_OVERFLOW) return fail(SOMA_EOVERFLOW, "a 16-bit occupation number reached 0xC000");
   if (err & ERR_TIMEOUT) return fail(SOMA_ETIMEOUT, "a bounded device wait gave up");
   return SOMA_OK;
-}
-
-soma_status sync(soma_t* h) {
-  SOMA_CUDA(cudaStreamSynchronize(h->stream));
-  return check_sticky(h);
 }
 
 soma_status update_fields(soma_t* h) {
@@ -783,8 +781,10 @@ soma_status soma_get_positions(soma_t* h, float* dst, size_t n, int dst_on_devic
   if (!h || !dst) return fail(SOMA_EINVAL, "NULL argument");
   if (n != 3 * h->M) return fail(SOMA_EINVAL, "n=%zu, expected 3*M=%llu", n, (unsigned long long)(3 * h->M));
   const cudaMemcpyKind k = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  for (int d = 0; d < 3; ++d)
-    SOMA_CUDA(cudaMemcpyAsync(dst + d * h->M, h->pos + d * h->plane, sizeof(float) * h->M, k, h->stream));
+  const bool one = h->plane == h->M;   // planes without padding: one copy
+  for (int d = 0; d < (one ? 1 : 3); ++d)
+    SOMA_CUDA(cudaMemcpyAsync(dst + d * h->M, h->pos + d * h->plane,
+                              sizeof(float) * (one ? 3 * h->M : h->M), k, h->stream));
   return sync(h);
 }
 
