@@ -171,6 +171,18 @@ __device__ __forceinline__ unsigned long long f2_fma_rn(unsigned long long a, un
   return d;
 }
 
+__device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul_rn(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_both(float v) { return f2_pack(v, v); }
+
 // Philox4x32-10 with the round keys taken from the kernel parameters (the
 // key schedule is the same for every thread, so it is computed once on the
 // host and read from the constant bank).

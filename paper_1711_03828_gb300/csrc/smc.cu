@@ -20,13 +20,6 @@
 
 namespace soma {
 
-__device__ __forceinline__ void cell3(const Geom& g, float x, float y, float z, uint32_t& cx,
-                                      uint32_t& cy, uint32_t& cz) {
-  cx = fold_axis(g, 0, x, (uint32_t)g.nx);
-  cy = fold_axis(g, 1, y, (uint32_t)g.ny);
-  cz = fold_axis(g, 2, z, (uint32_t)g.nz);
-}
-
 // omega at the cell and minus its central-difference gradient (the field force).
 template <typename WT>
 __device__ __forceinline__ float field_and_force(const Geom& g, const WT* w, uint32_t cx, uint32_t cy,
@@ -121,23 +114,26 @@ struct SmcSlot {
   uint32_t c;         // old cell
 };
 
-__device__ __forceinline__ SmcSlot smc_slot(const Geom& g, const float4* tab, float x, float y, float z,
-                                            uint64_t m, uint32_t sweep, uint32_t ctr3a,
-                                            bool valid, uint32_t* first_word) {
-  SmcSlot q;
-  q.x = x; q.y = y; q.z = z;
-  // the old cell's table entry first: in flight during the draw and normals
-  uint32_t cx, cy, cz;
-  cell3(g, x, y, z, cx, cy, cz);
-  q.c = (cz * (uint32_t)g.ny + cy) * (uint32_t)g.nx + cx;
-  q.w = 0.f;
-  q.fx = q.fy = q.fz = 0.f;
-  if (valid) q.w = smc_field(tab, q.c, q.fx, q.fy, q.fz);
-  const uint4 r1 = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3a), g);
-  *first_word = r1.w;
-  smc_normals(r1, q.gx, q.gy, q.gz);
-  q.lnu = log_uniform_open(spare_uniform_word(r1));
-  return q;
+// The two slots of a lane, particles m and m + 1 of the draws' counters: the old
+// cells' table entries first (in flight during the draws and normals).
+__device__ __forceinline__ void smc_slots(const Geom& g, const float4* tab0, const float4* tab1,
+                                          uint64_t m, uint32_t sweep, uint32_t ctr3a, SmcSlot& q0,
+                                          SmcSlot& q1, uint32_t* first_word) {
+  // an empty slot's cell lies in the grid; its values are not used
+  q0.c = cell_of(g, q0.x, q0.y, q0.z);
+  q1.c = cell_of(g, q1.x, q1.y, q1.z);
+  q0.w = smc_field(tab0, q0.c, q0.fx, q0.fy, q0.fz);
+  q1.w = smc_field(tab1, q1.c, q1.fx, q1.fy, q1.fz);
+  const uint64_t m1 = m + 1u;
+  const uint4 r0 = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3a), g);
+  const uint4 r1 = philox_rk(make_uint4((uint32_t)m1, (uint32_t)(m1 >> 32), sweep, ctr3a), g);
+  *first_word = r0.w;
+  float n0[3], n1[3];
+  smc_normals2(r0, r1, n0, n1);
+  q0.gx = n0[0]; q0.gy = n0[1]; q0.gz = n0[2];
+  q1.gx = n1[0]; q1.gy = n1[1]; q1.gz = n1[2];
+  q0.lnu = log_uniform_open(spare_uniform_word(r0));
+  q1.lnu = log_uniform_open(spare_uniform_word(r1));
 }
 
 // One smart Monte Carlo move of M against the fixed partner sum
@@ -149,11 +145,9 @@ __device__ __forceinline__ bool smc_move(const SweepArgs& p, const float4* tab, 
   const float tx = __fadd_rn(M.x, fmaf(s2A, M.gx, A * Fx));
   const float ty = __fadd_rn(M.y, fmaf(s2A, M.gy, A * Fy));
   const float tz = __fadd_rn(M.z, fmaf(s2A, M.gz, A * Fz));
-  uint32_t cx, cy, cz;
-  cell3(p.g, tx, ty, tz, cx, cy, cz);
-  const uint32_t cn = (cz * (uint32_t)p.g.ny + cy) * (uint32_t)p.g.nx + cx;
-  float fnx = 0.f, fny = 0.f, fnz = 0.f, w_new = 0.f;
-  if (valid) w_new = smc_field(tab, cn, fnx, fny, fnz);
+  const uint32_t cn = cell_of(p.g, tx, ty, tz);
+  float fnx, fny, fnz;
+  const float w_new = smc_field(tab, cn, fnx, fny, fnz);
   const float dx = tx - M.x, dy = ty - M.y, dz = tz - M.z;
   const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
   const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -199,11 +193,12 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
   const float4* tab0 = p.smc_tab + (L.v0 == 1u ? 0u : p.g.cells);   // table plane of slot 0
   const float4* tab1 = p.smc_tab + (L.v1 == 1u ? 0u : p.g.cells);
   const uint32_t TN = p.G * p.g.N;
+  const uint32_t dense_tiles = TN == 64u ? (uint32_t)p.full_tiles : 0u;   // all lanes hold a pair
   unsigned my_acc = 0;
   // positions of the warp's next tile, loaded while the current one is moved
   float2 nx = make_float2(0.f, 0.f), ny = nx, nz = nx;
   auto load_pos = [&](uint32_t t) {
-    if (t < t_end && L.in_tile(t < (uint32_t)p.full_tiles, p.last_rows)) {
+    if (t < t_end && (t < dense_tiles || L.in_tile(t < (uint32_t)p.full_tiles, p.last_rows))) {
       const uint32_t b = t * TN + L.li0;
       nx = __ldcs(reinterpret_cast<const float2*>(p.x + b));
       ny = __ldcs(reinterpret_cast<const float2*>(p.y + b));
@@ -213,7 +208,7 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
   uint32_t tile = claim();
   load_pos(tile);
   while (tile < t_end) {
-    const bool valid = L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
+    const bool valid = tile < dense_tiles || L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
     const uint32_t base = tile * TN + L.li0;
     float2 px = make_float2(0.f, 0.f), py = px, pz = px;
     if (valid) {
@@ -223,10 +218,12 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
     }
     const uint32_t next_tile = claim();
     load_pos(next_tile);
-    uint32_t w0, w1;
+    uint32_t w0;
     const uint32_t cbase = base + (uint32_t)p.g.id_base;
-    const SmcSlot s0 = smc_slot(p.g, tab0, px.x, py.x, pz.x, cbase, sweep, ctr3a, valid, &w0);
-    const SmcSlot s1 = smc_slot(p.g, tab1, px.y, py.y, pz.y, cbase + 1u, sweep, ctr3a, valid, &w1);
+    SmcSlot s0, s1;
+    s0.x = px.x; s0.y = py.x; s0.z = pz.x;
+    s1.x = px.y; s1.y = py.y; s1.z = pz.y;
+    smc_slots(p.g, tab0, tab1, cbase, sweep, ctr3a, s0, s1, &w0);
     const bool sw = p.set_order_random && (__shfl_sync(FULL, w0, L.first_lane) & 1u);
     SmcSlot A = sw ? s1 : s0, B = sw ? s0 : s1;
     const float4* tA = sw ? tab1 : tab0;
@@ -302,8 +299,10 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_strip_kernel(const SweepArgs
     const float4* tR = aR ? tabA : tabB;
     uint32_t w;
     const uint64_t m = (uint64_t)(s.m + (IDX)p.g.id_base);
-    SmcSlot L = smc_slot(p.g, tL, v.Lx, v.Ly, v.Lz, m - 1u, sweep, ctr3, s.vL, &w);
-    SmcSlot R = smc_slot(p.g, tR, v.Rx, v.Ry, v.Rz, m, sweep, ctr3, s.vR, &w);
+    SmcSlot L, R;
+    L.x = v.Lx; L.y = v.Ly; L.z = v.Lz;
+    R.x = v.Rx; R.y = v.Ry; R.z = v.Rz;
+    smc_slots(p.g, tL, tR, m - 1u, sweep, ctr3, L, R, &w);
     {  // first set: R moves against L of its own and of the next unit
       const float qx = strip_next(L.x, nv.Lx, lane), qy = strip_next(L.y, nv.Ly, lane),
                   qz = strip_next(L.z, nv.Lz, lane);
