@@ -66,6 +66,7 @@ soma_status cuda_fail(cudaError_t e, const char* what) {
   } while (0)
 
 constexpr uint32_t GRAPH_CHUNK = 16;
+constexpr uint32_t RESIDENT_CYCLES = 4096;
 constexpr uint64_t MAX_M = 1ull << 40;
 // Supported position range |x|, |y|, |z| < 2^18 dL (exact cell fold).
 constexpr uint64_t POS_LIMIT = 1ull << 18;
@@ -90,10 +91,13 @@ struct soma_t {
   uint64_t plane = 0;  // floats per position plane (padded)
   float* pos = nullptr;
   uint32_t* n[2] = {nullptr, nullptr};
+  uint32_t* n_spare = nullptr;               // third count buffer of a resident system
+  ResidentShape resident{0, 0};              // many cycles per launch (resident.cu)
   void* w[2] = {nullptr, nullptr};
   unsigned long long* d_counters = nullptr;  // [0] sweep, [1] accepted
   unsigned* d_err = nullptr;                 // [0] error bits, [1] arrival counter,
-                                             // [2] range flag of soma_set_positions
+                                             // [2] range flag of soma_set_positions,
+                                             // [3] grid barrier of a resident launch
   double* d_scratch = nullptr;
   float4* d_smc = nullptr;                   // smart Monte Carlo table, smc_planes * cells, SMC only
   uint32_t smc_planes = 0;                   // one float4 plane per type (A, B or n_t types)
@@ -261,6 +265,7 @@ void release(soma_t* h) {
   cudaFree(h->pos);
   cudaFree(h->n[0]);
   cudaFree(h->n[1]);
+  cudaFree(h->n_spare);
   cudaFree(h->w[0]);
   cudaFree(h->w[1]);
   cudaFree(h->d_counters);
@@ -576,7 +581,7 @@ soma_status soma_create(const soma_system_desc* desc, soma_t** out) {
   ALLOC(h->w[0], wb * cells);
   ALLOC(h->w[1], wb * cells);
   ALLOC(h->d_counters, sizeof(unsigned long long) * 2);
-  ALLOC(h->d_err, sizeof(unsigned) * 3);
+  ALLOC(h->d_err, sizeof(unsigned) * 4);
   ALLOC(h->d_scratch, sizeof(double) * (h->scratch_doubles + 64));
   ALLOC(h->mlp_w, sizeof(float) * SOMA_MLP_PARAMS);
   ALLOC(h->mlp_q, 2 * SOMA_MLP_PARAMS);
@@ -594,11 +599,17 @@ soma_status soma_create(const soma_system_desc* desc, soma_t** out) {
                          (desc->flags & SOMA_FLAG_LEARNED_UMMA) != 0,
                          desc->set_order == SOMA_ITERATION_MOLECULE);
   h->plain_shape = sweep_shape(h->g, h->sm_count, h->grid_dtype, SOMA_MOVE_UNIFORM);
+  if (desc->n_chains_total == 0) h->resident = resident_shape(h->shape, h->sm_count);
+  if (h->resident.grid) {
+    e = cudaMalloc((void**)&h->n_spare, sizeof(uint32_t) * cells);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->n_spare, 0, sizeof(uint32_t) * cells, h->stream);
+    if (e != cudaSuccess) { release(h); return cuda_fail(e, "third count buffer"); }
+  }
 #define CK(call) do { e = (call); if (e != cudaSuccess) { release(h); return cuda_fail(e, #call); } } while (0)
   CK(cudaMemsetAsync(h->n[0], 0, sizeof(uint32_t) * cells, h->stream));
   CK(cudaMemsetAsync(h->n[1], 0, sizeof(uint32_t) * cells, h->stream));
   CK(cudaMemsetAsync(h->d_counters, 0, sizeof(unsigned long long) * 2, h->stream));
-  CK(cudaMemsetAsync(h->d_err, 0, sizeof(unsigned) * 3, h->stream));
+  CK(cudaMemsetAsync(h->d_err, 0, sizeof(unsigned) * 4, h->stream));
   CK(cudaMemsetAsync(h->mlp_w, 0, sizeof(float) * SOMA_MLP_PARAMS, h->stream));
   CK(cudaMemsetAsync(h->mlp_q, 0, 2 * SOMA_MLP_PARAMS, h->stream));
   CK(cudaMemsetAsync(h->mlp_m, 0, sizeof(float) * SOMA_MLP_PARAMS, h->stream));
@@ -648,6 +659,27 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
   if (h->n_types && !h->has_topo)
     return fail(SOMA_ESTATE, "n_t types take the architecture path: call soma_set_topology");
   uint32_t done = 0;
+  // a small system under uniform moves of linear chains: one launch for up to
+  // RESIDENT_CYCLES cycles (per-kernel timing needs the two kernels)
+  if (h->resident.grid && !h->timing && !h->has_topo && !h->n_types) {
+    for (; done < n;) {
+      ResidentArgs a;
+      a.s = sweep_args(h, h->shape);
+      a.f = field_args(h, 1);
+      a.n2 = h->n_spare;
+      a.bar = h->d_err + 3;
+      a.arrive = h->d_err + 1;
+      a.cycles = std::min(n - done, RESIDENT_CYCLES);
+      const cudaError_t e = launch_resident(a, h->resident, h->grid_dtype, h->stream);
+      if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
+      ++h->launches;
+      h->t.sweep_launches += a.cycles;
+      h->t.field_launches += a.cycles;
+      h->host_sweep += a.cycles;
+      done += a.cycles;
+    }
+    return SOMA_OK;
+  }
   if (!h->timing && n >= GRAPH_CHUNK) {
     if (!h->graph) {
       soma_status st = build_graph(h);

@@ -81,6 +81,11 @@ template <> __device__ __forceinline__ float load_w<__half>(const __half* p, uin
   return __half2float(__ldg(p + i));
 }
 
+template <typename WT> __device__ __forceinline__ float load_cvt(WT v);
+template <> __device__ __forceinline__ float load_cvt<float>(float v) { return v; }
+template <> __device__ __forceinline__ float load_cvt<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
+template <> __device__ __forceinline__ float load_cvt<__half>(__half v) { return __half2float(v); }
+
 template <typename WT> __device__ __forceinline__ WT store_cvt(float v);
 template <> __device__ __forceinline__ float store_cvt<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 store_cvt<__nv_bfloat16>(float v) {

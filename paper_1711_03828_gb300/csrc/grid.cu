@@ -6,6 +6,7 @@
 //   - energies: Eq. (h-bond), (V-harmonic), (discrete-ham); S(q): Sec. 5.6.
 #include "kernels.h"
 #include "draws.cuh"
+#include "omega.cuh"
 #include "square_sum.cuh"
 
 namespace soma {
@@ -131,18 +132,8 @@ __global__ void __launch_bounds__(256) fields_kernel(const FieldArgs p, unsigned
     const uint32_t v = nr[c];
     nc[c] = 0u;
     const uint32_t a = v & 0xFFFFu, b = v >> 16;
-    const float phiA = (float)a * p.inv_rho;
-    const float phiB = (float)b * p.inv_rho;
-    const float comp = p.kappa0 * (phiA + phiB - 1.f);
-    float wa, wb;
-    if (p.hamiltonian) {          // K^1: + chi_0 phi_k of the other type
-      wa = fmaf(2.f * p.half_chi0, phiB, comp);
-      wb = fmaf(2.f * p.half_chi0, phiA, comp);
-    } else {                      // K^0: -/+ chi_0/2 (phi_A - phi_B)
-      const float d = p.half_chi0 * (phiA - phiB);
-      wa = comp - d;
-      wb = comp + d;
-    }
+    float wa = omega_of(v, false, p.inv_rho, p.kappa0, p.half_chi0, p.hamiltonian);
+    float wb = omega_of(v, true, p.inv_rho, p.kappa0, p.half_chi0, p.hamiltonian);
     if (p.ext) {
       wa += p.ext[c];
       wb += p.ext[p.g.cells + c];

@@ -36,6 +36,27 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move,
 cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int grid_dtype,
                                  cudaStream_t st);
 
+// Many cycles of a small system in one cooperative launch (resident.cu).
+// grid 0: the system takes the two-kernel cycle.
+struct ResidentShape {
+  int grid, block;
+};
+struct ResidentArgs {
+  SweepArgs s;
+  FieldArgs f;
+  uint32_t* n2;        // third count buffer, cleared between launches
+  unsigned* bar;       // grid barrier counter, 0 between launches
+  unsigned* arrive;    // blocks that have ended, 0 between launches
+  uint32_t cycles;
+};
+// Largest system of the resident sweep, in tiles of 64 slots per SM: two tiles for
+// each of 24 warps.  Measured per cycle, resident against two kernels a cycle:
+// 40 tiles per SM 8.3 / 10.8 us, 91 tiles 14.6 / 14.4, 162 tiles 20.1 / 19.2.
+constexpr uint64_t RESIDENT_TILES_PER_SM = 48;
+ResidentShape resident_shape(const SweepShape& s, int sm_count);
+cudaError_t launch_resident(const ResidentArgs& a, const ResidentShape& s, int grid_dtype,
+                            cudaStream_t st);
+
 cudaError_t launch_init(const Geom& g, float* x, float* y, float* z, double sigma, int sm_count,
                         cudaStream_t st);
 // Re-label whole chains in Morton order of the 8^3-cell block of their first

@@ -58,6 +58,10 @@ struct PairLane {
     return li0 < (full ? tile_rows : last_rows);
   }
 
+  // omega of slot 0's / slot 1's type at cell c
+  __device__ __forceinline__ float field0(uint32_t c) const { return load_w<WT>(w0, c); }
+  __device__ __forceinline__ float field1(uint32_t c) const { return load_w<WT>(w1, c); }
+
   // Types of the two slots (true: B): field planes and count increments.
   __device__ __forceinline__ void set_types(bool b0, bool b1, const void* wA, const void* wB) {
     w0 = static_cast<const WT*>(b0 ? wB : wA);
@@ -91,8 +95,8 @@ struct PairState {
   bool valid;
 };
 
-template <typename WT, typename IDX, bool WIDE>
-__device__ __forceinline__ void pair_prepare(const Geom& g, const Geom& keys, const PairLane<WT>& L,
+template <typename LANE, typename IDX, bool WIDE>
+__device__ __forceinline__ void pair_prepare(const Geom& g, const Geom& keys, const LANE& L,
                                              IDX cbase, bool valid, uint32_t sweep, uint32_t ctr3,
                                              float a, float x0, float x1, float y0, float y1,
                                              float z0, float z1, PairState& P) {
@@ -108,8 +112,8 @@ __device__ __forceinline__ void pair_prepare(const Geom& g, const Geom& keys, co
   P.c1 = cell_of_floor_bits<WIDE>(g, __float_as_uint(fx1), __float_as_uint(fy1), __float_as_uint(fz1));
   P.wo0 = P.wo1 = 0.f;
   if (valid) {
-    P.wo0 = load_w<WT>(L.w0, P.c0);
-    P.wo1 = load_w<WT>(L.w1, P.c1);
+    P.wo0 = L.field0(P.c0);
+    P.wo1 = L.field1(P.c1);
   }
   const uint32_t hi = sizeof(IDX) > 4 ? (uint32_t)((uint64_t)cbase >> 32) : 0u;
   const uint4 r0 = philox_rk(make_uint4((uint32_t)cbase, hi, sweep, ctr3), keys);
@@ -140,8 +144,8 @@ __device__ __forceinline__ void pair_prepare(const Geom& g, const Geom& keys, co
   P.cn1 = cell_of_floor_bits<WIDE>(g, __float_as_uint(gx1), __float_as_uint(gy1), __float_as_uint(gz1));
   P.wn0 = P.wn1 = 0.f;
   if (valid) {
-    P.wn0 = load_w<WT>(L.w0, P.cn0);
-    P.wn1 = load_w<WT>(L.w1, P.cn1);
+    P.wn0 = L.field0(P.cn0);
+    P.wn1 = L.field1(P.cn1);
   }
   P.x0 = x0; P.x1 = x1; P.y0 = y0; P.y1 = y1; P.z0 = z0; P.z1 = z1;
   P.u0 = r0.w;
@@ -149,13 +153,20 @@ __device__ __forceinline__ void pair_prepare(const Geom& g, const Geom& keys, co
   P.valid = valid;
 }
 
-// Returns this lane's accepted moves.
-template <typename WT, typename IDX>
-__device__ __forceinline__ unsigned pair_finish(const PairLane<WT>& L, float* __restrict__ px,
+// The pair's positions after a cycle whose caller keeps them (resident.cu).
+struct PairEnd {
+  float2 x, y, z;
+  bool store;   // write them to memory as well
+};
+
+// Returns this lane's accepted moves.  KEEP: end receives the final positions,
+// which are stored only if end.store.
+template <typename LANE, typename IDX, bool KEEP>
+__device__ __forceinline__ unsigned pair_finish(const LANE& L, float* __restrict__ px,
                                                 float* __restrict__ py, float* __restrict__ pz,
                                                 uint32_t* __restrict__ nacc, IDX base,
                                                 const PairState& P, bool set_order_random,
-                                                float K1) {
+                                                float K1, PairEnd* end) {
   const bool valid = P.valid;
   const float K2 = 2.f * K1;
   const float x0 = P.x0, x1 = P.x1, y0 = P.y0, y1 = P.y1, z0 = P.z0, z1 = P.z1;
@@ -225,10 +236,17 @@ __device__ __forceinline__ unsigned pair_finish(const PairLane<WT>& L, float* __
     acc_count += acc;
   }
 
+  if (KEEP) {
+    end->x = sw ? make_float2(Bx, Ax) : make_float2(Ax, Bx);
+    end->y = sw ? make_float2(By, Ay) : make_float2(Ay, By);
+    end->z = sw ? make_float2(Bz, Az) : make_float2(Az, Bz);
+  }
   if (valid) {
-    __stcs(reinterpret_cast<float2*>(px + base), sw ? make_float2(Bx, Ax) : make_float2(Ax, Bx));
-    __stcs(reinterpret_cast<float2*>(py + base), sw ? make_float2(By, Ay) : make_float2(Ay, By));
-    __stcs(reinterpret_cast<float2*>(pz + base), sw ? make_float2(Bz, Az) : make_float2(Az, Bz));
+    if (!KEEP || end->store) {
+      __stcs(reinterpret_cast<float2*>(px + base), sw ? make_float2(Bx, Ax) : make_float2(Ax, Bx));
+      __stcs(reinterpret_cast<float2*>(py + base), sw ? make_float2(By, Ay) : make_float2(Ay, By));
+      __stcs(reinterpret_cast<float2*>(pz + base), sw ? make_float2(Bz, Az) : make_float2(Az, Bz));
+    }
     // one atomic when both end in the same cell, else one each
     const uint32_t vA = sw ? L.v1 : L.v0, vB = sw ? L.v0 : L.v1;
     const bool same = cA == cB;
@@ -247,9 +265,10 @@ __device__ __forceinline__ unsigned pair_tile(const Geom& g, const Geom& keys, c
                                               float K1, float x0, float x1, float y0, float y1,
                                               float z0, float z1) {
   PairState P;
-  pair_prepare<WT, IDX, WIDE>(g, keys, L, cbase, PARTIAL ? valid : true, sweep, ctr3, a, x0, x1, y0,
-                              y1, z0, z1, P);
-  return pair_finish<WT, IDX>(L, px, py, pz, nacc, base, P, set_order_random, K1);
+  pair_prepare<PairLane<WT>, IDX, WIDE>(g, keys, L, cbase, PARTIAL ? valid : true, sweep, ctr3, a, x0,
+                                        x1, y0, y1, z0, z1, P);
+  return pair_finish<PairLane<WT>, IDX, false>(L, px, py, pz, nacc, base, P, set_order_random, K1,
+                                               nullptr);
 }
 
 }  // namespace soma
