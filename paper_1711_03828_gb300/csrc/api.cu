@@ -310,6 +310,8 @@ FieldArgs field_args(soma_t* h, int after_sweep) {
   f.hamiltonian = (int)h->desc.hamiltonian;
   f.ext = h->has_ext ? h->d_ext : nullptr;
   f.forbidden = h->has_forbidden ? h->d_forbidden : nullptr;
+  f.tab = h->d_smc;
+  f.tab_kind = FIELD_FORCE;
   return f;
 }
 
@@ -417,21 +419,15 @@ TypesArgs types_args(soma_t* h, int after_sweep) {
   return a;
 }
 
-// the table of fields and field forces that smart Monte Carlo sweeps read,
-// after every field update of such a system (A and B, or one plane per type)
-cudaError_t launch_smc_table_of(soma_t* h) {
-  if (!h->d_smc) return cudaSuccess;
-  ++h->launches;
-  if (h->n_types)
-    return launch_smc_table_planes(h->g, h->wt, h->n_types, h->d_smc, h->sm_count, h->stream);
-  return launch_smc_table(h->g, h->w[0], h->w[1], h->d_smc, h->grid_dtype, h->sm_count, h->stream);
-}
-
-// the field update of one cycle: the packed A | B grid or the type planes
+// the field update of one cycle: the packed A | B grid (with the table of a smart
+// Monte Carlo system) or the type planes and their table
 cudaError_t launch_fields_any(soma_t* h, const FieldArgs& fa, const TypesArgs& ta) {
-  cudaError_t e = h->n_types ? launch_fields_types(ta, h->d_err + 1, h->sm_count, h->stream)
-                             : launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream);
-  if (e == cudaSuccess) e = launch_smc_table_of(h);
+  if (!h->n_types) return launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream);
+  cudaError_t e = launch_fields_types(ta, h->d_err + 1, h->sm_count, h->stream);
+  if (e == cudaSuccess && h->d_smc) {
+    ++h->launches;
+    e = launch_smc_table_planes(h->g, h->wt, h->n_types, h->d_smc, h->sm_count, h->stream);
+  }
   return e;
 }
 
@@ -502,9 +498,8 @@ soma_status update_fields(soma_t* h) {
     SOMA_CUDA(cudaMemsetAsync(nn, 0, sizeof(uint32_t) * h->n_types * h->g.cells, h->stream));
     SOMA_CUDA(launch_histogram_types(h->g, h->x(), h->y(), h->z(), h->d_topo_ttab, h->d_arch, nn,
                                      h->sm_count, h->stream));
-    SOMA_CUDA(launch_fields_types(types_args(h, 0), h->d_err + 1, h->sm_count, h->stream));
+    SOMA_CUDA(launch_fields_any(h, field_args(h, 0), types_args(h, 0)));
     h->launches += 2;
-    SOMA_CUDA(launch_smc_table_of(h));
     return SOMA_OK;
   }
   // count into n[s&1] (cleared first), then omega from it
@@ -514,10 +509,8 @@ soma_status update_fields(soma_t* h) {
                              h->d_seq, h->d_seq ? h->d_arch : nullptr,
                              h->has_topo ? h->d_topo_len : nullptr));
   ++h->launches;
-  const FieldArgs fa = field_args(h, 0);
-  SOMA_CUDA(launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream));
+  SOMA_CUDA(launch_fields_any(h, field_args(h, 0), types_args(h, 0)));
   ++h->launches;
-  SOMA_CUDA(launch_smc_table_of(h));
   return SOMA_OK;
 }
 
@@ -687,7 +680,7 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
     }
     while (n - done >= GRAPH_CHUNK) {
       SOMA_CUDA(cudaGraphLaunch(h->graph, h->stream));
-      h->launches += (h->d_smc ? 3 : 2) * GRAPH_CHUNK;
+      h->launches += (h->d_smc && h->n_types ? 3 : 2) * GRAPH_CHUNK;
       h->t.sweep_launches += GRAPH_CHUNK;
       h->t.field_launches += GRAPH_CHUNK;
       h->host_sweep += GRAPH_CHUNK;
@@ -759,8 +752,7 @@ soma_status soma_shard_fields(soma_t* h, const uint32_t* summed, size_t cells) {
   SOMA_CUDA(cudaMemcpyAsync(nn, summed, sizeof(uint32_t) * cells, cudaMemcpyDefault, h->stream));
   const FieldArgs fa = field_args(h, after_sweep);
   st = timed(h, 1, [&] {
-    cudaError_t e = launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream);
-    return e == cudaSuccess ? launch_smc_table_of(h) : e;
+    return launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream);
   });
   if (st != SOMA_OK) return st;
   if (after_sweep) ++h->host_sweep;
@@ -1503,11 +1495,14 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
   std::vector<float> hJ(cfg->batch), hla(cfg->batch);
   double first = 0.0, last = 0.0, acc_last = 0.0;
   const SweepArgs sa = sweep_args(h, h->plain_shape);
-  const FieldArgs fa = field_args(h, 1);
+  FieldArgs fa = field_args(h, 1);
+  float4* const tab = fa.tab;
   for (uint32_t k = 0; k < cfg->steps; ++k) {
     // trajectories of the plain method
     for (uint32_t c = 0; c < cfg->sweeps_between; ++c) {
       SOMA_CUDA(launch_sweep_uniform(sa, h->plain_shape, h->grid_dtype, h->stream));
+      // the table of the handle's own move belongs to the last fields
+      fa.tab = k + 1 == cfg->steps && c + 1 == cfg->sweeps_between ? tab : nullptr;
       SOMA_CUDA(launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream));
       ++h->host_sweep;
       h->launches += 2;

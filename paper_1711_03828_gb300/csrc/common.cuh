@@ -279,7 +279,10 @@ struct FieldArgs {
   int hamiltonian;          // 0: K^0_inter, 1: K^1_inter
   const float* ext;         // external potential, A cells then B cells (or NULL)
   const uint8_t* forbidden; // cells no particle may enter (or NULL)
+  float4* tab;              // table of a force-biased or learned sweep (or NULL), what it holds
+  int tab_kind;
 };
+constexpr int FIELD_ONLY = 0, FIELD_FORCE = 1, FIELD_GRADIENT = 2;
 
 // One system of a batch (device table entry).
 struct BatchSys {

@@ -132,12 +132,9 @@ constexpr int MOL_BLOCK = 128;
 const void* molecule_kernel_ptr(uint32_t N, int grid_dtype, size_t* smem, bool prepare);
 // smart Monte Carlo sweep kernel: pair tiles or strips (big: 64-bit indices)
 const void* smc_kernel_ptr(bool strip, bool big);
-// Smart Monte Carlo table (omega and the central-difference field force per
-// type and cell, float4, A then B) from the omega planes of storage type
-// grid_dtype; rebuilt after every field update of a smart Monte Carlo system.
-cudaError_t launch_smc_table(const Geom& g, const void* wA, const void* wB, float4* tab,
-                             int grid_dtype, int sm_count, cudaStream_t st);
-// the same for n_t types: one float4 plane per type from the FP32 planes w
+// Smart Monte Carlo table for n_t types (omega and the central-difference field
+// force per cell, one float4 plane per type) from the FP32 planes w, rebuilt after
+// every field update; two types have theirs from the field kernel
 cudaError_t launch_smc_table_planes(const Geom& g, const float* w, uint32_t planes, float4* tab,
                                     int sm_count, cudaStream_t st);
 

@@ -35,28 +35,9 @@ __device__ __forceinline__ float field_and_force(const Geom& g, const WT* w, uin
   return load_w<WT>(w, row + cx);
 }
 
-// The smart Monte Carlo table, rebuilt after every field update: per type and
-// cell, omega_t(c) and minus its central difference along each axis (the
-// field force of field_and_force, bit for bit), one float4 per cell, A then
-// B.  A move reads it with one 16-byte load at its old and one at its trial
-// cell instead of gathering seven field values at each.
-template <typename WT>
-__global__ void smc_table_kernel(const Geom g, const WT* __restrict__ wA, const WT* __restrict__ wB,
-                                 float4* __restrict__ tab) {
-  const uint32_t nx = g.nx, ny = g.ny;
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < g.cells;
-       c += gridDim.x * blockDim.x) {
-    const uint32_t cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
-    float fx, fy, fz;
-    float w = field_and_force<WT>(g, wA, cx, cy, cz, fx, fy, fz);
-    tab[c] = make_float4(w, fx, fy, fz);
-    w = field_and_force<WT>(g, wB, cx, cy, cz, fx, fy, fz);
-    tab[g.cells + c] = make_float4(w, fx, fy, fz);
-  }
-}
-
-// The same table for n_t types: one plane of float4 per type from the FP32
-// field planes w (n_types * cells).
+// The table of a smart Monte Carlo sweep for n_t types (of two types: made by the
+// field kernel): one plane of float4 per type, omega and the field force, from
+// the FP32 field planes w (n_types * cells).
 __global__ void smc_table_planes_kernel(const Geom g, const float* __restrict__ w, uint32_t planes,
                                         float4* __restrict__ tab) {
   const uint32_t nx = g.nx, ny = g.ny;
@@ -74,25 +55,6 @@ __global__ void smc_table_planes_kernel(const Geom g, const float* __restrict__ 
 cudaError_t launch_smc_table_planes(const Geom& g, const float* w, uint32_t planes, float4* tab,
                                     int sm_count, cudaStream_t st) {
   smc_table_planes_kernel<<<4 * sm_count, 256, 0, st>>>(g, w, planes, tab);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_smc_table(const Geom& g, const void* wA, const void* wB, float4* tab,
-                             int grid_dtype, int sm_count, cudaStream_t st) {
-  const int grid = 4 * sm_count;
-  switch (grid_dtype) {
-    case 1:
-      smc_table_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
-          g, static_cast<const __nv_bfloat16*>(wA), static_cast<const __nv_bfloat16*>(wB), tab);
-      break;
-    case 2:
-      smc_table_kernel<__half><<<grid, 256, 0, st>>>(g, static_cast<const __half*>(wA),
-                                                     static_cast<const __half*>(wB), tab);
-      break;
-    default:
-      smc_table_kernel<float><<<grid, 256, 0, st>>>(g, static_cast<const float*>(wA),
-                                                    static_cast<const float*>(wB), tab);
-  }
   return cudaGetLastError();
 }
 
