@@ -311,7 +311,7 @@ FieldArgs field_args(soma_t* h, int after_sweep) {
   f.ext = h->has_ext ? h->d_ext : nullptr;
   f.forbidden = h->has_forbidden ? h->d_forbidden : nullptr;
   f.tab = h->d_smc;
-  f.tab_kind = FIELD_FORCE;
+  f.tab_kind = h->desc.move == SOMA_MOVE_LEARNED ? FIELD_GRADIENT : FIELD_FORCE;
   return f;
 }
 
@@ -591,6 +591,10 @@ soma_status soma_create(const soma_system_desc* desc, soma_t** out) {
                          (desc->flags & SOMA_FLAG_LEARNED_FP32) != 0,
                          (desc->flags & SOMA_FLAG_LEARNED_UMMA) != 0,
                          desc->set_order == SOMA_ITERATION_MOLECULE);
+  if (h->shape.learned_tc) {
+    e = cudaMalloc((void**)&h->d_smc, sizeof(float4) * 4 * cells);
+    if (e != cudaSuccess) { release(h); return cuda_fail(e, "gradient table"); }
+  }
   h->plain_shape = sweep_shape(h->g, h->sm_count, h->grid_dtype, SOMA_MOVE_UNIFORM);
   if (desc->n_chains_total == 0) h->resident = resident_shape(h->shape, h->sm_count);
   if (h->resident.grid) {

@@ -122,7 +122,7 @@ cudaError_t launch_adam(float* w, float* m, float* v, const float* grad, void* w
                         float b1, float b2, float eps, int step, float inv_n, cudaStream_t st);
 cudaError_t launch_quantize(const float* w, void* wq, cudaStream_t st);
 const void* learned_kernel_ptr(int Q, int grid_dtype);
-const void* learned_tc_kernel_ptr(int grid_dtype, bool umma);
+const void* learned_tc_kernel_ptr(bool umma);
 // one warp waits (at most limit polls) for an mbarrier phase nobody completes
 cudaError_t launch_wait_probe(uint32_t limit, unsigned* err, cudaStream_t st);
 // molecule-parallel sweep kernel for chains of N particles (one thread per

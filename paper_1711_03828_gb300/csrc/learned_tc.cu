@@ -28,11 +28,16 @@ namespace soma {
 
 constexpr int TC_W1 = 0, TC_B1 = 384, TC_W2 = 416, TC_B2 = 1440, TC_W3 = 1472, TC_B3 = 1600;
 
+// The network as mma.sync operand fragments, by lane, in shared memory: one copy
+// for the block's warps.  Held in registers (46 of them per thread) the kernel ran
+// at 12 warps per SM; each evaluation reads its fragments once for both 16-row
+// halves of the warp's rows.
 struct MlpFrag {
-  uint32_t w1[4][2];     // layer 1, n-tile x (k 0-7 | k 8-15)
-  uint32_t w2[2][4][2];  // layer 2, k-step x n-tile
-  uint32_t w3[2][2];     // layer 3, k-step
-  float b1[4][2], b2[4][2], b3[2];
+  uint4 w1[4][32];    // layer 1 per n-tile: k 0-7, k 8-15, bias pair
+  uint4 w2[4][32];    // layer 2 per n-tile: k-steps 0 and 1
+  uint4 w3[32];       // layer 3: k-steps 0 and 1
+  float2 b2[4][32];   // bias pairs of layers 2 and 3 (zeros past output 3)
+  float2 b3[32];
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -58,34 +63,38 @@ __device__ __forceinline__ void mma16816(float d[4], const uint32_t a[4], const 
 
 __device__ __forceinline__ float wv(const __nv_bfloat16* W, int idx) { return __bfloat162float(W[idx]); }
 
-// Fragments of this lane: g = lane/4 (row / output column group), c = lane%4.
-__device__ __forceinline__ void mlp_load(MlpFrag& R, const __nv_bfloat16* __restrict__ W, int lane) {
-  const int g = lane >> 2, c = lane & 3;
-#pragma unroll
-  for (int nt = 0; nt < 4; ++nt) {
+// Fills R with the block's threads; lane: g = lane/4 (row / output column group),
+// c = lane%4.
+__device__ __forceinline__ void mlp_load(MlpFrag& R, const __nv_bfloat16* __restrict__ W) {
+  for (int k = threadIdx.x; k < 4 * 32; k += blockDim.x) {
+    const int nt = k >> 5, lane = k & 31, g = lane >> 2, c = lane & 3;
     const int j = 8 * nt + g;  // output unit (column of B)
     const int k0 = 2 * c, k1 = 2 * c + 8;
-    R.w1[nt][0] = pack_bf16(wv(W, TC_W1 + 12 * j + k0), wv(W, TC_W1 + 12 * j + k0 + 1));
-    R.w1[nt][1] = (k1 < 12) ? pack_bf16(wv(W, TC_W1 + 12 * j + k1), wv(W, TC_W1 + 12 * j + k1 + 1)) : 0u;
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const int kk = 16 * ks + 2 * c;
-      R.w2[ks][nt][0] = pack_bf16(wv(W, TC_W2 + 32 * j + kk), wv(W, TC_W2 + 32 * j + kk + 1));
-      R.w2[ks][nt][1] = pack_bf16(wv(W, TC_W2 + 32 * j + kk + 8), wv(W, TC_W2 + 32 * j + kk + 9));
+    uint4 v;
+    v.x = pack_bf16(wv(W, TC_W1 + 12 * j + k0), wv(W, TC_W1 + 12 * j + k0 + 1));
+    v.y = (k1 < 12) ? pack_bf16(wv(W, TC_W1 + 12 * j + k1), wv(W, TC_W1 + 12 * j + k1 + 1)) : 0u;
+    v.z = __float_as_uint(wv(W, TC_B1 + 8 * nt + 2 * c));
+    v.w = __float_as_uint(wv(W, TC_B1 + 8 * nt + 2 * c + 1));
+    R.w1[nt][lane] = v;
+    const int kk = 2 * c;
+    v.x = pack_bf16(wv(W, TC_W2 + 32 * j + kk), wv(W, TC_W2 + 32 * j + kk + 1));
+    v.y = pack_bf16(wv(W, TC_W2 + 32 * j + kk + 8), wv(W, TC_W2 + 32 * j + kk + 9));
+    v.z = pack_bf16(wv(W, TC_W2 + 32 * j + kk + 16), wv(W, TC_W2 + 32 * j + kk + 17));
+    v.w = pack_bf16(wv(W, TC_W2 + 32 * j + kk + 24), wv(W, TC_W2 + 32 * j + kk + 25));
+    R.w2[nt][lane] = v;
+    R.b2[nt][lane] = make_float2(wv(W, TC_B2 + 8 * nt + 2 * c), wv(W, TC_B2 + 8 * nt + 2 * c + 1));
+    if (nt == 0) {
+      v = make_uint4(0u, 0u, 0u, 0u);
+      if (g < 4) {
+        v.x = pack_bf16(wv(W, TC_W3 + 32 * g + kk), wv(W, TC_W3 + 32 * g + kk + 1));
+        v.y = pack_bf16(wv(W, TC_W3 + 32 * g + kk + 8), wv(W, TC_W3 + 32 * g + kk + 9));
+        v.z = pack_bf16(wv(W, TC_W3 + 32 * g + kk + 16), wv(W, TC_W3 + 32 * g + kk + 17));
+        v.w = pack_bf16(wv(W, TC_W3 + 32 * g + kk + 24), wv(W, TC_W3 + 32 * g + kk + 25));
+      }
+      R.w3[lane] = v;
+      R.b3[lane] = c < 2 ? make_float2(wv(W, TC_B3 + 2 * c), wv(W, TC_B3 + 2 * c + 1)) : make_float2(0.f, 0.f);
     }
-    R.b1[nt][0] = wv(W, TC_B1 + 8 * nt + 2 * c);
-    R.b1[nt][1] = wv(W, TC_B1 + 8 * nt + 2 * c + 1);
-    R.b2[nt][0] = wv(W, TC_B2 + 8 * nt + 2 * c);
-    R.b2[nt][1] = wv(W, TC_B2 + 8 * nt + 2 * c + 1);
   }
-#pragma unroll
-  for (int ks = 0; ks < 2; ++ks) {
-    const int kk = 16 * ks + 2 * c;
-    R.w3[ks][0] = g < 4 ? pack_bf16(wv(W, TC_W3 + 32 * g + kk), wv(W, TC_W3 + 32 * g + kk + 1)) : 0u;
-    R.w3[ks][1] = g < 4 ? pack_bf16(wv(W, TC_W3 + 32 * g + kk + 8), wv(W, TC_W3 + 32 * g + kk + 9)) : 0u;
-  }
-  R.b3[0] = c < 2 ? wv(W, TC_B3 + 2 * c) : 0.f;
-  R.b3[1] = c < 2 ? wv(W, TC_B3 + 2 * c + 1) : 0.f;
 }
 
 // Network outputs for this lane's feature vector f; every lane of the warp
@@ -114,51 +123,61 @@ __device__ __forceinline__ void mlp_warp(const MlpFrag& R, __nv_bfloat16* sf, fl
                  : "=r"(a1[mt][0]), "=r"(a1[mt][1]), "=r"(a1[mt][2]), "=r"(a1[mt][3])
                  : "r"(addr));
   }
-  // layer 1 -> ReLU -> layer 2 operands
+  // layer 1 -> ReLU -> layer 2 operands, both row halves per fragment read
   uint32_t a2[2][2][4];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    float d[4][4];
+  for (int ks = 0; ks < 2; ++ks) {
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      const float cb[4] = {R.b1[nt][0], R.b1[nt][1], R.b1[nt][0], R.b1[nt][1]};
-      mma16816(d[nt], a1[mt], R.w1[nt], cb);
-    }
+    for (int h = 0; h < 2; ++h) {
+      const uint4 w = R.w1[2 * ks + h][lane];
+      const uint32_t wb[2] = {w.x, w.y};
+      const float cb[4] = {__uint_as_float(w.z), __uint_as_float(w.w), __uint_as_float(w.z),
+                           __uint_as_float(w.w)};
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      a2[mt][ks][0] = relu_pack(d[2 * ks][0], d[2 * ks][1]);
-      a2[mt][ks][1] = relu_pack(d[2 * ks][2], d[2 * ks][3]);
-      a2[mt][ks][2] = relu_pack(d[2 * ks + 1][0], d[2 * ks + 1][1]);
-      a2[mt][ks][3] = relu_pack(d[2 * ks + 1][2], d[2 * ks + 1][3]);
+      for (int mt = 0; mt < 2; ++mt) {
+        float d[4];
+        mma16816(d, a1[mt], wb, cb);
+        a2[mt][ks][2 * h] = relu_pack(d[0], d[1]);
+        a2[mt][ks][2 * h + 1] = relu_pack(d[2], d[3]);
+      }
     }
   }
-  // layer 2 -> ReLU -> layer 3 -> outputs
+  // layer 2 -> ReLU -> layer 3 operands
+  uint32_t a3[2][2][4];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    float d[4][4];
+  for (int ks = 0; ks < 2; ++ks) {
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      const float cb[4] = {R.b2[nt][0], R.b2[nt][1], R.b2[nt][0], R.b2[nt][1]};
-      mma16816(d[nt], a2[mt][0], R.w2[0][nt], cb);
-      mma16816(d[nt], a2[mt][1], R.w2[1][nt], d[nt]);
+    for (int h = 0; h < 2; ++h) {
+      const uint4 w = R.w2[2 * ks + h][lane];
+      const float2 bv = R.b2[2 * ks + h][lane];
+      const uint32_t w0[2] = {w.x, w.y}, w1[2] = {w.z, w.w};
+      const float cb[4] = {bv.x, bv.y, bv.x, bv.y};
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt) {
+        float d[4];
+        mma16816(d, a2[mt][0], w0, cb);
+        mma16816(d, a2[mt][1], w1, d);
+        a3[mt][ks][2 * h] = relu_pack(d[0], d[1]);
+        a3[mt][ks][2 * h + 1] = relu_pack(d[2], d[3]);
+      }
     }
-    uint32_t a3[2][4];
+  }
+  {
+    const uint4 w = R.w3[lane];
+    const float2 bv = R.b3[lane];
+    const uint32_t w0[2] = {w.x, w.y}, w1[2] = {w.z, w.w};
+    const float cb[4] = {bv.x, bv.y, bv.x, bv.y};
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      a3[ks][0] = relu_pack(d[2 * ks][0], d[2 * ks][1]);
-      a3[ks][1] = relu_pack(d[2 * ks][2], d[2 * ks][3]);
-      a3[ks][2] = relu_pack(d[2 * ks + 1][0], d[2 * ks + 1][1]);
-      a3[ks][3] = relu_pack(d[2 * ks + 1][2], d[2 * ks + 1][3]);
-    }
-    float e[4];
-    const float cb[4] = {R.b3[0], R.b3[1], R.b3[0], R.b3[1]};
-    mma16816(e, a3[0], R.w3[0], cb);
-    mma16816(e, a3[1], R.w3[1], e);
-    if (c < 2) {
-      so[4 * (16 * mt + g) + 2 * c] = e[0];
-      so[4 * (16 * mt + g) + 2 * c + 1] = e[1];
-      so[4 * (16 * mt + g + 8) + 2 * c] = e[2];
-      so[4 * (16 * mt + g + 8) + 2 * c + 1] = e[3];
+    for (int mt = 0; mt < 2; ++mt) {
+      float e[4];
+      mma16816(e, a3[mt][0], w0, cb);
+      mma16816(e, a3[mt][1], w1, e);
+      if (c < 2) {
+        so[4 * (16 * mt + g) + 2 * c] = e[0];
+        so[4 * (16 * mt + g) + 2 * c + 1] = e[1];
+        so[4 * (16 * mt + g + 8) + 2 * c] = e[2];
+        so[4 * (16 * mt + g + 8) + 2 * c + 1] = e[3];
+      }
     }
   }
   __syncwarp();
@@ -355,42 +374,34 @@ struct UmmaNet {
   }
 };
 
-// Interpolated field gradient at (x,y,z) and omega of its cell (as learned.cu).
-template <typename WT>
-__device__ __forceinline__ float grad_at(const Geom& g, const WT* w, float x, float y, float z,
-                                         float gr[3], uint32_t* cell) {
+// Interpolated field gradient at (x,y,z) and omega of its cell (the values of
+// learned.cu's interp_gradient) from the table entry of the cell in the plane
+// of the particle's type: one 32-byte sector instead of seven gathered field
+// values and the index arithmetic of six neighbours.
+__device__ __forceinline__ float grad_at(const Geom& g, const float4* __restrict__ tab, float x,
+                                         float y, float z, float gr[3], uint32_t* cell) {
   const uint32_t cx = fold_axis(g, 0, x, (uint32_t)g.nx);
   const uint32_t cy = fold_axis(g, 1, y, (uint32_t)g.ny);
   const uint32_t cz = fold_axis(g, 2, z, (uint32_t)g.nz);
-  const uint32_t nx = g.nx, ny = g.ny, nz = g.nz;
-  const uint32_t c = (cz * ny + cy) * nx + cx;
-  const uint32_t xm = cx == 0 ? nx - 1 : cx - 1, xp = cx + 1 == nx ? 0 : cx + 1;
-  const uint32_t ym = cy == 0 ? ny - 1 : cy - 1, yp = cy + 1 == ny ? 0 : cy + 1;
-  const uint32_t zm = cz == 0 ? nz - 1 : cz - 1, zp = cz + 1 == nz ? 0 : cz + 1;
-  const float w0 = load_w<WT>(w, c);
-  const float lo0 = w0 - load_w<WT>(w, (cz * ny + cy) * nx + xm);
-  const float lo1 = w0 - load_w<WT>(w, (cz * ny + ym) * nx + cx);
-  const float lo2 = w0 - load_w<WT>(w, (zm * ny + cy) * nx + cx);
-  const float hi0 = load_w<WT>(w, (cz * ny + cy) * nx + xp) - w0;
-  const float hi1 = load_w<WT>(w, (cz * ny + yp) * nx + cx) - w0;
-  const float hi2 = load_w<WT>(w, (zp * ny + cy) * nx + cx) - w0;
-  gr[0] = fmaf(x - floorf(x), hi0 - lo0, lo0);
-  gr[1] = fmaf(y - floorf(y), hi1 - lo1, lo1);
-  gr[2] = fmaf(z - floorf(z), hi2 - lo2, lo2);
+  const uint32_t c = (cz * (uint32_t)g.ny + cy) * (uint32_t)g.nx + cx;
+  const float4 q = __ldg(tab + 2u * c), d = __ldg(tab + 2u * c + 1u);
+  gr[0] = fmaf(x - floorf(x), d.x, q.y);
+  gr[1] = fmaf(y - floorf(y), d.y, q.z);
+  gr[2] = fmaf(z - floorf(z), d.z, q.w);
   *cell = c;
-  return w0;
+  return q.x;
 }
 
 // One learned move of this lane's mover r (partners pv, nv when hp, hn).
-template <typename WT, typename Net>
-__device__ __forceinline__ bool learned_move(const Geom& g, Net& net, const WT* wt, bool isA,
+template <typename Net>
+__device__ __forceinline__ bool learned_move(const Geom& g, Net& net, const float4* wt, bool isA,
                                              bool hp, bool hn, float& rx, float& ry, float& rz,
                                              uint32_t& cell, float px, float py, float pz, float qx,
                                              float qy, float qz, const float xi[3], float lnu,
                                              float sigma0, float K_b, bool valid) {
   float f[12], gr[3], o[4], orv[4];
   uint32_t c_old, c_new;
-  const float w_old = grad_at<WT>(g, wt, rx, ry, rz, gr, &c_old);
+  const float w_old = grad_at(g, wt, rx, ry, rz, gr, &c_old);
   f[0] = hp ? rx - px : 0.f; f[1] = hp ? ry - py : 0.f; f[2] = hp ? rz - pz : 0.f;
   f[3] = hn ? qx - rx : 0.f; f[4] = hn ? qy - ry : 0.f; f[5] = hn ? qz - rz : 0.f;
   f[6] = gr[0]; f[7] = gr[1]; f[8] = gr[2];
@@ -402,7 +413,7 @@ __device__ __forceinline__ bool learned_move(const Geom& g, Net& net, const WT* 
   const float tx = __fadd_rn(rx, fmaf(sig, xi[0], o[0]));
   const float ty = __fadd_rn(ry, fmaf(sig, xi[1], o[1]));
   const float tz = __fadd_rn(rz, fmaf(sig, xi[2], o[2]));
-  const float w_new = grad_at<WT>(g, wt, tx, ty, tz, gr, &c_new);
+  const float w_new = grad_at(g, wt, tx, ty, tz, gr, &c_new);
   f[0] = hp ? tx - px : 0.f; f[1] = hp ? ty - py : 0.f; f[2] = hp ? tz - pz : 0.f;
   f[3] = hn ? qx - tx : 0.f; f[4] = hn ? qy - ty : 0.f; f[5] = hn ? qz - tz : 0.f;
   f[6] = gr[0]; f[7] = gr[1]; f[8] = gr[2];
@@ -433,23 +444,34 @@ __device__ __forceinline__ bool learned_move(const Geom& g, Net& net, const WT* 
   return acc;
 }
 
+// Positions of a lane's pair in a tile (zeros where it has none).
+struct PairPos {
+  float2 x, y, z;
+};
+__device__ __forceinline__ PairPos load_pair(const SweepArgs& p, uint32_t base, bool valid) {
+  PairPos v;
+  v.x = v.y = v.z = make_float2(0.f, 0.f);
+  if (valid) {
+    v.x = __ldcs(reinterpret_cast<const float2*>(p.x + base));
+    v.y = __ldcs(reinterpret_cast<const float2*>(p.y + base));
+    v.z = __ldcs(reinterpret_cast<const float2*>(p.z + base));
+  }
+  return v;
+}
+
 // One tile of the paired learned sweep for this lane (particles base, base+1);
 // valid: this lane's pair exists.  Returns the accepted moves.
-template <typename WT, typename Net>
-__device__ __forceinline__ unsigned learned_pair_tile(const SweepArgs& p, const PairLane<WT>& L,
+template <typename Net>
+__device__ __forceinline__ unsigned learned_pair_tile(const SweepArgs& p, const PairLane<float>& L,
                                                       Net& net, uint32_t* __restrict__ nacc,
                                                       uint32_t base, bool valid, uint32_t sweep,
-                                                      bool A0, bool A1) {
+                                                      bool A0, bool A1, const PairPos& at) {
   const int lane = L.lane;
   const uint32_t ctr3a = (PURPOSE_MOVE << 24) | (p.g.replica & 0xFFFFFFu);
   const uint32_t ctr3b = (PURPOSE_MOVE2 << 24) | (p.g.replica & 0xFFFFFFu);
-  float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f, z0 = 0.f, z1 = 0.f;
-  if (valid) {
-    const float2 a = __ldcs(reinterpret_cast<const float2*>(p.x + base));
-    const float2 b = __ldcs(reinterpret_cast<const float2*>(p.y + base));
-    const float2 c = __ldcs(reinterpret_cast<const float2*>(p.z + base));
-    x0 = a.x; x1 = a.y; y0 = b.x; y1 = b.y; z0 = c.x; z1 = c.y;
-  }
+  float x0 = at.x.x, x1 = at.x.y, y0 = at.y.x, y1 = at.y.y, z0 = at.z.x, z1 = at.z.y;
+  const float4* tab0 = p.smc_tab + (A0 ? 0u : 2u * (size_t)p.g.cells);   // plane of slot 0
+  const float4* tab1 = p.smc_tab + (A1 ? 0u : 2u * (size_t)p.g.cells);
   // normals by Box-Muller with the hardware log and sincos: the acceptance
   // uses the realised trial position, so the move stays exact
   float xi0[3], xi1[3], lnu0, lnu1;
@@ -496,7 +518,7 @@ __device__ __forceinline__ unsigned learned_pair_tile(const SweepArgs& p, const 
     const float px = odd ? x0 : sx, py = odd ? y0 : sy, pz = odd ? z0 : sz;
     const float qx = odd ? sx : x1, qy = odd ? sy : y1, qz = odd ? sz : z1;
     uint32_t cell;
-    const bool acc = learned_move<WT, Net>(p.g, net, odd ? L.w1 : L.w0, odd ? A1 : A0, hp, hn, rx,
+    const bool acc = learned_move<Net>(p.g, net, odd ? tab1 : tab0, odd ? A1 : A0, hp, hn, rx,
                                            ry, rz, cell, px, py, pz, qx, qy, qz,
                                            odd ? xi1 : xi0, odd ? lnu1 : lnu0, p.learned_sigma0,
                                            p.K_b, valid);
@@ -518,32 +540,45 @@ __device__ __forceinline__ unsigned learned_pair_tile(const SweepArgs& p, const 
   return n_acc;
 }
 
-// mma.sync network: every warp walks its own tiles.
-template <typename WT>
-__global__ void __launch_bounds__(128) sweep_learned_tc_kernel(const SweepArgs p,
-                                                               const __nv_bfloat16* __restrict__ wq) {
-  __shared__ __align__(16) __nv_bfloat16 s_feat[4][32 * 16];
-  __shared__ __align__(16) float s_out[4][32 * 4];
+// mma.sync network: every warp takes tiles of its block's contiguous range from
+// a shared-memory counter (one block of 16 warps per SM, 128 registers; with the
+// fragments in registers 12 warps, 20 and 24 warps spill and gain nothing).
+// 67M particles of N = 64: 3.11 ms a cycle before, 2.62-2.68 now (the field and
+// gradient table 0.06 of it); 1M: 54.5 and 49.1 us.
+constexpr int TC_WARPS = 16;
+__global__ void __launch_bounds__(32 * TC_WARPS, 1)
+    sweep_learned_tc_kernel(const SweepArgs p, const __nv_bfloat16* __restrict__ wq) {
+  __shared__ __align__(16) __nv_bfloat16 s_feat[TC_WARPS][32 * 16];
+  __shared__ __align__(16) float s_out[TC_WARPS][32 * 4];
+  __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  MlpFrag R;
-  mlp_load(R, wq, lane);
-  WarpNet net{&R, s_feat[wib], s_out[wib], lane};
+  __shared__ MlpFrag s_frag;
+  mlp_load(s_frag, wq);
+  WarpNet net{&s_frag, s_feat[wib], s_out[wib], lane};
   const uint32_t n_tiles_all = (uint32_t)p.n_tiles;
   const uint32_t chunk = (n_tiles_all + gridDim.x - 1) / gridDim.x;
   const uint32_t t_begin = blockIdx.x * chunk;
   const uint32_t t_end = min(t_begin + chunk, n_tiles_all);
+  if (threadIdx.x == 0) s_next = 0u;
+  __syncthreads();
+  auto claim = [&]() -> uint32_t {
+    uint32_t t = 0u;
+    if (lane == 0) t = atomicAdd(&s_next, 1u);
+    return t_begin + __shfl_sync(FULL, t, 0);
+  };
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
-  PairLane<WT> L;
+  PairLane<float> L;
   L.init(lane, p.g.N, p.g.N_A, p.wA, p.wB);
-  const uint32_t ci0 = L.li0 % p.g.N;
-  const bool A0 = ci0 < p.g.N_A, A1 = ci0 + 1 < p.g.N_A;
+  const bool A0 = L.ci0 < p.g.N_A, A1 = L.ci0 + 1 < p.g.N_A;
   const uint32_t TN = p.G * p.g.N;
   unsigned my_acc = 0;
-  for (uint32_t tile = t_begin + wib; tile < t_end; tile += 4) {
+  for (uint32_t tile = claim(); tile < t_end; tile = claim()) {
     const bool valid = L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
-    my_acc += learned_pair_tile<WT, WarpNet>(p, L, net, nacc, tile * TN + L.li0, valid, sweep, A0, A1);
+    const uint32_t base = tile * TN + L.li0;
+    my_acc += learned_pair_tile<WarpNet>(p, L, net, nacc, base, valid, sweep, A0, A1,
+                                         load_pair(p, base, valid));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
@@ -553,7 +588,6 @@ __global__ void __launch_bounds__(128) sweep_learned_tc_kernel(const SweepArgs p
 // tcgen05 network: the block's four warps step through their tiles together
 // (every network evaluation is one block-wide M = 128 product); a warp
 // without a tile of its own takes part with empty rows.
-template <typename WT>
 __global__ void __launch_bounds__(128) sweep_learned_umma_kernel(const SweepArgs p,
                                                                  const __nv_bfloat16* __restrict__ wq) {
   __shared__ UmmaSmem sm;
@@ -602,17 +636,17 @@ __global__ void __launch_bounds__(128) sweep_learned_umma_kernel(const SweepArgs
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
-  PairLane<WT> L;
+  PairLane<float> L;
   L.init(lane, p.g.N, p.g.N_A, p.wA, p.wB);
-  const uint32_t ci0 = L.li0 % p.g.N;
-  const bool A0 = ci0 < p.g.N_A, A1 = ci0 + 1 < p.g.N_A;
+  const bool A0 = L.ci0 < p.g.N_A, A1 = L.ci0 + 1 < p.g.N_A;
   const uint32_t TN = p.G * p.g.N;
   unsigned my_acc = 0;
   for (uint32_t r = 0; r < rounds; ++r) {
     const uint32_t tile = t_begin + 4 * r + (uint32_t)wib;
     const bool valid = tile < t_end && L.in_tile(tile < (uint32_t)p.full_tiles, p.last_rows);
     const uint32_t base = (tile < t_end ? tile : t_begin) * TN + L.li0;
-    my_acc += learned_pair_tile<WT, UmmaNet>(p, L, net, nacc, base, valid && net.ok, sweep, A0, A1);
+    my_acc += learned_pair_tile<UmmaNet>(p, L, net, nacc, base, valid && net.ok, sweep, A0, A1,
+                                         load_pair(p, base, valid && net.ok));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
@@ -650,14 +684,8 @@ cudaError_t launch_wait_probe(uint32_t limit, unsigned* err, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-const void* learned_tc_kernel_ptr(int grid_dtype, bool umma) {
-  if (umma)
-    return grid_dtype == 1 ? (const void*)sweep_learned_umma_kernel<__nv_bfloat16>
-         : grid_dtype == 2 ? (const void*)sweep_learned_umma_kernel<__half>
-                           : (const void*)sweep_learned_umma_kernel<float>;
-  return grid_dtype == 1 ? (const void*)sweep_learned_tc_kernel<__nv_bfloat16>
-       : grid_dtype == 2 ? (const void*)sweep_learned_tc_kernel<__half>
-                         : (const void*)sweep_learned_tc_kernel<float>;
+const void* learned_tc_kernel_ptr(bool umma) {
+  return umma ? (const void*)sweep_learned_umma_kernel : (const void*)sweep_learned_tc_kernel;
 }
 
 }  // namespace soma

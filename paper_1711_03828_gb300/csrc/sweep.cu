@@ -333,7 +333,7 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   if (move == 2 && s.pair && !s.big && !learned_fp32) {
     s.learned_tc = true;
     s.learned_umma = learned_umma;
-    s.block = 128;
+    s.block = learned_umma ? 128 : 512;   // one block of 12 warps per SM (mma.sync)
   } else if (molecule && move == 0) {
     s.molecule = true;
     s.block = MOL_BLOCK;
@@ -342,16 +342,17 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   }
   s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
   s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
-  const void* fn = s.learned_tc ? learned_tc_kernel_ptr(grid_dtype, s.learned_umma)
+  const void* fn = s.learned_tc ? learned_tc_kernel_ptr(s.learned_umma)
                  : s.molecule   ? molecule_kernel_ptr(N, grid_dtype, &s.smem, true)
                                 : sweep_kernel_ptr(s, grid_dtype, false);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, s.smem);
   if (per_sm < 1) per_sm = 1;
   const uint64_t warps_per_block = (uint64_t)s.block / 32;
-  // a strip launch spreads its items over all SMs, however few they are
+  // strips and learned tiles are spread over all SMs, however few they are
   const uint64_t need = s.molecule ? (n_chains + s.block - 1) / s.block
                       : s.strip    ? s.n_items
+                      : s.learned_tc && !s.learned_umma ? s.n_tiles
                                    : (s.n_tiles + warps_per_block - 1) / warps_per_block;
   const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
   s.grid = (int)(need < cap ? need : cap);
