@@ -34,6 +34,14 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
   return c;
 }
 
+// First statement of the kernels of a cycle (launch_chained): lets the next kernel
+// of the stream be set up while this one runs, and waits until the one before
+// has ended and its writes are visible.
+__device__ __forceinline__ void chained_begin() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Symmetric uniform (2k+1)/2^24 - 1 of the top 24 bits k of r: never 0, and
 // exact in FP32: k*2^-23 + (2^-24 - 1) is representable, and the fused
 // multiply-add rounds the exact value once.

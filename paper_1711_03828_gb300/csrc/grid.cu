@@ -135,6 +135,7 @@ cudaError_t launch_range_check(const float* p, uint64_t n, float lim, unsigned* 
 // divisions per cell.
 template <typename WT, int TAB, bool PLAIN>
 __global__ void __launch_bounds__(256) fields_kernel(const FieldArgs p, unsigned* arrive) {
+  chained_begin();
   const unsigned long long s = *p.d_sweep;
   const int rd = p.after_sweep ? (int)((s + 1ull) & 1ull) : (int)(s & 1ull);
   const uint32_t* __restrict__ nr = rd ? p.n1 : p.n0;
@@ -211,12 +212,14 @@ __global__ void __launch_bounds__(256) fields_kernel(const FieldArgs p, unsigned
 }
 
 template <typename WT, bool PLAIN>
-static void launch_fields_as(const FieldArgs& a, unsigned* arrive, unsigned blocks, cudaStream_t st) {
-  switch (a.tab ? a.tab_kind : FIELD_ONLY) {
-    case FIELD_FORCE: fields_kernel<WT, FIELD_FORCE, PLAIN><<<blocks, 256, 0, st>>>(a, arrive); break;
-    case FIELD_GRADIENT: fields_kernel<WT, FIELD_GRADIENT, PLAIN><<<blocks, 256, 0, st>>>(a, arrive); break;
-    default: fields_kernel<WT, FIELD_ONLY, PLAIN><<<blocks, 256, 0, st>>>(a, arrive); break;
-  }
+static const void* fields_ptr_of(int tab_kind) {
+  return tab_kind == FIELD_FORCE      ? (const void*)fields_kernel<WT, FIELD_FORCE, PLAIN>
+         : tab_kind == FIELD_GRADIENT ? (const void*)fields_kernel<WT, FIELD_GRADIENT, PLAIN>
+                                      : (const void*)fields_kernel<WT, FIELD_ONLY, PLAIN>;
+}
+template <typename WT>
+static const void* fields_ptr(int tab_kind, bool plain) {
+  return plain ? fields_ptr_of<WT, true>(tab_kind) : fields_ptr_of<WT, false>(tab_kind);
 }
 
 cudaError_t launch_fields(const FieldArgs& a, unsigned* arrive, int grid_dtype, int sm_count,
@@ -225,22 +228,13 @@ cudaError_t launch_fields(const FieldArgs& a, unsigned* arrive, int grid_dtype, 
   const uint64_t cap = (uint64_t)sm_count * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
+  const int kind = a.tab ? a.tab_kind : FIELD_ONLY;
   const bool plain = a.hamiltonian == 0 && !a.ext && !a.forbidden;
-  const unsigned nb = (unsigned)blocks;
-  switch (grid_dtype) {
-    case 1:
-      plain ? launch_fields_as<__nv_bfloat16, true>(a, arrive, nb, st)
-            : launch_fields_as<__nv_bfloat16, false>(a, arrive, nb, st);
-      break;
-    case 2:
-      plain ? launch_fields_as<__half, true>(a, arrive, nb, st)
-            : launch_fields_as<__half, false>(a, arrive, nb, st);
-      break;
-    default:
-      plain ? launch_fields_as<float, true>(a, arrive, nb, st)
-            : launch_fields_as<float, false>(a, arrive, nb, st);
-  }
-  return cudaGetLastError();
+  const void* fn = grid_dtype == 1   ? fields_ptr<__nv_bfloat16>(kind, plain)
+                   : grid_dtype == 2 ? fields_ptr<__half>(kind, plain)
+                                     : fields_ptr<float>(kind, plain);
+  void* args[] = {const_cast<FieldArgs*>(&a), &arrive};
+  return launch_chained(fn, dim3((unsigned)blocks), dim3(256), args, 0, st);
 }
 
 template <typename WT>

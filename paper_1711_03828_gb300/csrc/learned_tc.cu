@@ -553,6 +553,7 @@ __global__ void __launch_bounds__(32 * TC_WARPS, 1)
   __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   __shared__ MlpFrag s_frag;
+  chained_begin();
   mlp_load(s_frag, wq);
   WarpNet net{&s_frag, s_feat[wib], s_out[wib], lane};
   const uint32_t n_tiles_all = (uint32_t)p.n_tiles;

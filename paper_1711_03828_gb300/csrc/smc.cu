@@ -40,6 +40,7 @@ __device__ __forceinline__ float field_and_force(const Geom& g, const WT* w, uin
 // the FP32 field planes w (n_types * cells).
 __global__ void smc_table_planes_kernel(const Geom g, const float* __restrict__ w, uint32_t planes,
                                         float4* __restrict__ tab) {
+  chained_begin();
   const uint32_t nx = g.nx, ny = g.ny;
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < g.cells;
        c += gridDim.x * blockDim.x) {
@@ -54,8 +55,8 @@ __global__ void smc_table_planes_kernel(const Geom g, const float* __restrict__ 
 
 cudaError_t launch_smc_table_planes(const Geom& g, const float* w, uint32_t planes, float4* tab,
                                     int sm_count, cudaStream_t st) {
-  smc_table_planes_kernel<<<4 * sm_count, 256, 0, st>>>(g, w, planes, tab);
-  return cudaGetLastError();
+  void* args[] = {const_cast<Geom*>(&g), &w, &planes, &tab};
+  return launch_chained((const void*)smc_table_planes_kernel, dim3(4 * sm_count), dim3(256), args, 0, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
     if (lane == 0) t = atomicAdd(&s_next, 1u);
     return t_begin + __shfl_sync(FULL, t, 0);
   };
+  chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_strip_kernel(const SweepArgs
   const uint32_t item0 = blockIdx.x * chunk;
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;

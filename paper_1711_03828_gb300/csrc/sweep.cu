@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(768, 1) sweep_strip_kernel(const SweepArgs p) 
   const uint32_t item0 = blockIdx.x * chunk;
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(768, 1) sweep_pair_kernel(const SweepArgs p) {
     if (lane == 0) t = atomicAdd(&s_next, 1u);
     return t_begin + __shfl_sync(FULL, t, 0);
   };
+  chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = ((s64 + 1ull) & 1ull) ? p.n1 : p.n0;
@@ -366,7 +368,8 @@ cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int gr
   const void* fn = s.molecule ? molecule_kernel_ptr(a.g.N, grid_dtype, &smem, false)
                               : sweep_kernel_ptr(s, grid_dtype, a.seq != nullptr);
   void* args[] = {const_cast<SweepArgs*>(&a)};
-  return cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st);
+  return s.molecule ? cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st)
+                    : launch_chained(fn, dim3(s.grid), dim3(s.block), args, smem, st);
 }
 
 }  // namespace soma

@@ -504,6 +504,7 @@ __global__ void __launch_bounds__(768, 1) sweep_topology_pair_kernel(const TopoA
     if (lane == 0) v = atomicAdd(&s_next, 1u);
     return t_begin + __shfl_sync(FULL, v, 0);
   };
+  chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   uint32_t* __restrict__ nacc = MULTI ? (((s64 + 1ull) & 1ull) ? t.nt1 : t.nt0)
@@ -861,7 +862,7 @@ int topology_pair_grid(uint64_t n_mol, uint32_t G, int sm_count) {
 cudaError_t launch_sweep_topology_pair(const TopoArgs& a, int grid, int grid_dtype, cudaStream_t st,
                                        bool types, bool smc) {
   void* args[] = {const_cast<TopoArgs*>(&a)};
-  return cudaLaunchKernel(smc ? topology_pair_ptr_of<true>(grid_dtype, types)
+  return launch_chained(smc ? topology_pair_ptr_of<true>(grid_dtype, types)
                               : topology_pair_ptr_of<false>(grid_dtype, types),
                           dim3(grid), dim3(768), args, 0, st);
 }

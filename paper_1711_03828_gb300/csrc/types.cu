@@ -23,6 +23,7 @@ namespace {
 // next sweep counts into, writes every type's field; after a sweep the last
 // block to finish advances the device sweep counter (as fields_kernel does).
 __global__ void __launch_bounds__(256) fields_types_kernel(const TypesArgs p, unsigned* arrive) {
+  chained_begin();
   const unsigned long long s = *p.d_sweep;
   const int rd = p.after_sweep ? (int)((s + 1ull) & 1ull) : (int)(s & 1ull);
   const uint32_t* __restrict__ nr = rd ? p.n1 : p.n0;
@@ -185,8 +186,8 @@ cudaError_t launch_fields_types(const TypesArgs& a, unsigned* arrive, int sm_cou
   const uint64_t cap = (uint64_t)sm_count * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  fields_types_kernel<<<(unsigned)blocks, 256, 0, st>>>(a, arrive);
-  return cudaGetLastError();
+  void* args[] = {const_cast<TypesArgs*>(&a), &arrive};
+  return launch_chained((const void*)fields_types_kernel, dim3((unsigned)blocks), dim3(256), args, 0, st);
 }
 
 cudaError_t launch_histogram_types(const Geom& g, const float* x, const float* y, const float* z,
