@@ -434,8 +434,8 @@ cudaError_t launch_fields_any(soma_t* h, const FieldArgs& fa, const TypesArgs& t
 cudaError_t launch_sweep_any(soma_t* h, const SweepArgs& sa) {
   const bool types = h->n_types != 0;
   if (h->has_topo && h->shape.molecule)
-    return launch_molecule_topology(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->stream,
-                                    types);
+    return launch_molecule_topology(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->sm_count,
+                                    h->stream, types);
   if (h->has_topo && h->topo_R)
     return launch_sweep_topology_pair(topo_args(h, sa), h->topo_grid, h->grid_dtype, h->stream, types,
                                       h->desc.move == SOMA_MOVE_SMC);
@@ -444,7 +444,7 @@ cudaError_t launch_sweep_any(soma_t* h, const SweepArgs& sa) {
                                  h->stream, types, h->desc.move == SOMA_MOVE_SMC);
   if (h->desc.move == SOMA_MOVE_LEARNED)
     return launch_sweep_learned(sa, h->shape, h->grid_dtype, h->mlp_q, h->stream);
-  return launch_sweep_uniform(sa, h->shape, h->grid_dtype, h->stream);
+  return launch_sweep_uniform(sa, h->shape, h->grid_dtype, h->sm_count, h->stream);
 }
 
 soma_status one_cycle(soma_t* h) {
@@ -983,7 +983,8 @@ namespace {
 // launch grid of the architecture sweep for the handle's iteration, move and types
 void set_topo_grid(soma_t* h) {
   h->topo_grid = h->shape.molecule
-                     ? molecule_topology_grid(h->g.N, h->grid_dtype, h->sm_count, h->g.n_chains)
+                     ? molecule_topology_grid(h->g.N, h->grid_dtype, h->sm_count, h->g.n_chains,
+                                              h->n_types != 0)
                  : h->topo_R ? topology_pair_grid(h->g.n_chains, h->topo_G, h->sm_count)
                      : topology_grid(h->grid_dtype, h->shape.big, h->sm_count, h->shape.n_tiles,
                                      h->n_types != 0, h->desc.move == SOMA_MOVE_SMC);
@@ -1504,7 +1505,7 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
   for (uint32_t k = 0; k < cfg->steps; ++k) {
     // trajectories of the plain method
     for (uint32_t c = 0; c < cfg->sweeps_between; ++c) {
-      SOMA_CUDA(launch_sweep_uniform(sa, h->plain_shape, h->grid_dtype, h->stream));
+      SOMA_CUDA(launch_sweep_uniform(sa, h->plain_shape, h->grid_dtype, h->sm_count, h->stream));
       // the table of the handle's own move belongs to the last fields
       fa.tab = k + 1 == cfg->steps && c + 1 == cfg->sweeps_between ? tab : nullptr;
       SOMA_CUDA(launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream));

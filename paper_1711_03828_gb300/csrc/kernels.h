@@ -47,7 +47,6 @@ struct SweepShape {
   bool learned_tc;  // learned move with the network on the tensor cores
   bool learned_umma;  // ... through tcgen05 (else warp-level mma.sync)
   bool molecule;      // molecule-parallel iteration (one thread per chain)
-  size_t smem;        // dynamic shared memory of the sweep kernel
   int block;
   int grid;
 };
@@ -56,7 +55,7 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move,
                        bool learned_fp32 = false, bool learned_umma = false,
                        bool molecule = false);
 cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int grid_dtype,
-                                 cudaStream_t st);
+                                 int sm_count, cudaStream_t st);
 
 // Many cycles of a small system in one cooperative launch (resident.cu).
 // grid 0: the system takes the two-kernel cycle.
@@ -147,11 +146,12 @@ const void* learned_kernel_ptr(int Q, int grid_dtype);
 const void* learned_tc_kernel_ptr(bool umma);
 // one warp waits (at most limit polls) for an mbarrier phase nobody completes
 cudaError_t launch_wait_probe(uint32_t limit, unsigned* err, cudaStream_t st);
-// molecule-parallel sweep kernel for chains of N particles (one thread per
-// chain, MOL_BLOCK threads and chains per block); *smem receives its dynamic
-// shared memory (prepare: allow the kernel that much, once at create)
+// molecule-parallel sweep kernel for n_chains chains of N particles and its dynamic
+// shared memory; molecule_grid gives its blocks and allows it that memory (call
+// it before the first launch, outside stream capture)
 constexpr int MOL_BLOCK = 128;
-const void* molecule_kernel_ptr(uint32_t N, int grid_dtype, size_t* smem, bool prepare);
+const void* molecule_kernel(uint64_t n_chains, uint32_t N, int grid_dtype, int sm_count, size_t* smem);
+int molecule_grid(uint64_t n_chains, uint32_t N, int grid_dtype, int sm_count);
 // smart Monte Carlo sweep kernel: pair tiles or strips (big: 64-bit indices)
 const void* smc_kernel_ptr(bool strip, bool big);
 // Smart Monte Carlo table for n_t types (omega and the central-difference field
@@ -221,9 +221,9 @@ cudaError_t launch_sweep_topology(const TopoArgs& a, int grid, int grid_dtype, b
 // the molecule-parallel iteration for molecules of any architecture (N <= 64);
 // the grid helper also allows the kernel its shared memory (call it before
 // the first launch, outside stream capture)
-int molecule_topology_grid(uint32_t N, int grid_dtype, int sm_count, uint64_t n_chains);
-cudaError_t launch_molecule_topology(const TopoArgs& a, int grid, int grid_dtype, cudaStream_t st,
-                                     bool types = false);
+int molecule_topology_grid(uint32_t N, int grid_dtype, int sm_count, uint64_t n_chains, bool types);
+cudaError_t launch_molecule_topology(const TopoArgs& a, int grid, int grid_dtype, int sm_count,
+                                     cudaStream_t st, bool types);
 // out[0] = sum over the bonds of the architectures of |b|^2, out[1] = sum over
 // the molecules of |r_last - r_0|^2 with r_last the last particle of each
 // molecule's architecture (lengths alen) (FP64); part: 2 OBS_BLOCKS doubles

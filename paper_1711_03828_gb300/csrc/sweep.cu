@@ -318,7 +318,6 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   s.learned_tc = false;
   s.learned_umma = false;
   s.molecule = false;
-  s.smem = 0;
   s.Q = (N <= 64) ? 1 : (N <= 128 ? 2 : 4);
   s.G = (uint32_t)(64 * s.Q) / N;
   s.n_tiles = (n_chains + s.G - 1) / s.G;
@@ -345,15 +344,17 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
   s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
   const void* fn = s.learned_tc ? learned_tc_kernel_ptr(s.learned_umma)
-                 : s.molecule   ? molecule_kernel_ptr(N, grid_dtype, &s.smem, true)
                                 : sweep_kernel_ptr(s, grid_dtype, false);
+  if (s.molecule) {
+    s.grid = molecule_grid(n_chains, N, grid_dtype, sm_count);
+    return s;
+  }
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, s.smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, 0);
   if (per_sm < 1) per_sm = 1;
   const uint64_t warps_per_block = (uint64_t)s.block / 32;
   // strips and learned tiles are spread over all SMs, however few they are
-  const uint64_t need = s.molecule ? (n_chains + s.block - 1) / s.block
-                      : s.strip    ? s.n_items
+  const uint64_t need = s.strip    ? s.n_items
                       : s.learned_tc && !s.learned_umma ? s.n_tiles
                                    : (s.n_tiles + warps_per_block - 1) / warps_per_block;
   const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
@@ -363,9 +364,9 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
 }
 
 cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int grid_dtype,
-                                 cudaStream_t st) {
+                                 int sm_count, cudaStream_t st) {
   size_t smem = 0;
-  const void* fn = s.molecule ? molecule_kernel_ptr(a.g.N, grid_dtype, &smem, false)
+  const void* fn = s.molecule ? molecule_kernel(a.g.n_chains, a.g.N, grid_dtype, sm_count, &smem)
                               : sweep_kernel_ptr(s, grid_dtype, a.seq != nullptr);
   void* args[] = {const_cast<SweepArgs*>(&a)};
   return s.molecule ? cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st)
