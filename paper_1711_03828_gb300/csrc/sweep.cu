@@ -42,13 +42,13 @@ __device__ __forceinline__ float bond_change(bool hp, bool hq, float rx, float r
 }
 
 // Chains of odd length and of more than 64 particles, in the strips of
-// strip.cuh.  One block of 24 warps per SM owns a contiguous range of items,
+// strip.cuh.  One block of 32 warps per SM owns a contiguous range of items,
 // handed out from a shared-memory counter.  WIDE: every axis has two or more
 // cells.  Issue-bound like the paired kernel (454 warp instructions a strip);
 // the paper's thin film (N = 100, 16.5M particles, 16-bit fields): 214 us a
 // sweep in tiles of 128 slots, 152 us in strips.
 template <typename WT, typename IDX, bool WIDE>
-__global__ void __launch_bounds__(768, 1) sweep_strip_kernel(const SweepArgs p) {
+__global__ void __launch_bounds__(1024, 1) sweep_strip_kernel(const SweepArgs p) {
   __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
   const uint32_t chunk = (p.n_items + gridDim.x - 1) / gridDim.x;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(768, 1) sweep_strip_kernel(const SweepArgs p) 
 }
 
 // Even N <= 64: the paired tile body of pair_body.cuh over one system.  One
-// block of 24 warps per SM owns a contiguous range of tiles (spatially
+// block of 32 warps per SM owns a contiguous range of tiles (spatially
 // ordered chains); its warps take the range's tiles in order from a
 // shared-memory counter, so they work on neighbouring tiles (field values
 // repeat in L1) and all finish within a tile of each other.  With three
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(768, 1) sweep_strip_kernel(const SweepArgs p) 
 // MIXED: a mixture of linear architectures (the type sequence of each chain
 // is read per tile); otherwise every chain is the diblock of N_A A particles.
 template <typename WT, typename IDX, bool MIXED>
-__global__ void __launch_bounds__(768, 1) sweep_pair_kernel(const SweepArgs p) {
+__global__ void __launch_bounds__(1024, 1) sweep_pair_kernel(const SweepArgs p) {
   __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
   const uint32_t n_tiles_all = (uint32_t)p.n_tiles;
@@ -339,7 +339,10 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
     s.molecule = true;
     s.block = MOL_BLOCK;
   } else if (move != 2) {
-    s.block = 768;   // one block of 24 warps per SM
+    // one block per SM: 32 warps in 64 registers without spills for uniform moves
+    // (16 cycles of 134M particles with 24 warps 16.56 ms, 28 16.42, 32 16.22; thin
+    // film 2.61, 2.46, 2.43), 24 for smart Monte Carlo's 77 registers
+    s.block = move == 1 ? 768 : 1024;
   }
   s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
   s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
