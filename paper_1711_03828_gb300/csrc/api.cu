@@ -92,7 +92,7 @@ struct soma_t {
   float* pos = nullptr;
   uint32_t* n[2] = {nullptr, nullptr};
   uint32_t* n_spare = nullptr;               // third count buffer of a resident system
-  ResidentShape resident{0, 0};              // many cycles per launch (resident.cu)
+  ResidentShape resident{0, 0, 0};              // many cycles per launch (resident.cu)
   void* w[2] = {nullptr, nullptr};
   unsigned long long* d_counters = nullptr;  // [0] sweep, [1] accepted
   unsigned* d_err = nullptr;                 // [0] error bits, [1] arrival counter,
@@ -596,7 +596,8 @@ soma_status soma_create(const soma_system_desc* desc, soma_t** out) {
     if (e != cudaSuccess) { release(h); return cuda_fail(e, "gradient table"); }
   }
   h->plain_shape = sweep_shape(h->g, h->sm_count, h->grid_dtype, SOMA_MOVE_UNIFORM);
-  if (desc->n_chains_total == 0) h->resident = resident_shape(h->shape, h->sm_count);
+  if (desc->n_chains_total == 0) 
+    h->resident = resident_shape(h->shape, h->g.cells, h->grid_dtype, h->sm_count);
   if (h->resident.grid) {
     e = cudaMalloc((void**)&h->n_spare, sizeof(uint32_t) * cells);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->n_spare, 0, sizeof(uint32_t) * cells, h->stream);

@@ -61,6 +61,7 @@ cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int gr
 // grid 0: the system takes the two-kernel cycle.
 struct ResidentShape {
   int grid, block;
+  size_t cluster_smem;   // shared memory of the one-cluster kernel (0: the cooperative one)
 };
 struct ResidentArgs {
   SweepArgs s;
@@ -70,11 +71,18 @@ struct ResidentArgs {
   unsigned* arrive;    // blocks that have ended, 0 between launches
   uint32_t cycles;
 };
-// Largest system of the resident sweep, in tiles of 64 slots per SM: two tiles for
-// each of 24 warps.  Measured per cycle, resident against two kernels a cycle:
-// 40 tiles per SM 8.3 / 10.8 us, 91 tiles 14.6 / 14.4, 162 tiles 20.1 / 19.2.
-constexpr uint64_t RESIDENT_TILES_PER_SM = 48;
-ResidentShape resident_shape(const SweepShape& s, int sm_count);
+// Largest system of the resident sweep, in tiles of 64 slots per SM: three rounds of
+// 32 warps.  Resident against two kernels a cycle: 27 tiles per SM 7.1 and 9.5 us, 40
+// 8.7 and 11.9, 61 11.4 and 12.1, 91 13.8 and 14.1, 121 16.8 and 16.6, 162 19.3 and 19.2.
+constexpr uint64_t RESIDENT_TILES_PER_SM = 96;
+// One cluster: 16 blocks of up to 16 warps, a tile each, and the counts three times
+// in a block's shared memory (96 KB at the limit).  With 32 warps on its 16 SMs
+// their issue slots are the time: 32,768 particles 4.4 us a cycle against 4.2 over
+// all SMs; 13,664 2.9 against 3.9.
+constexpr int CLUSTER_BLOCKS = 16;
+constexpr int CLUSTER_WARPS = 16;
+constexpr uint32_t CLUSTER_CELLS = 8192;
+ResidentShape resident_shape(const SweepShape& s, uint32_t cells, int grid_dtype, int sm_count);
 cudaError_t launch_resident(const ResidentArgs& a, const ResidentShape& s, int grid_dtype,
                             cudaStream_t st);
 
