@@ -130,10 +130,11 @@ __device__ __forceinline__ bool smc_move(const SweepArgs& p, const float4* tab, 
   return acc;
 }
 
-// Paired smart Monte Carlo sweep (even N <= 64).  One block of 24 warps per
-// SM owns a contiguous range of tiles, which its warps take in order from a
+// Paired smart Monte Carlo sweep (even N <= 64).  One block of 28 warps per
+// SM (72 registers; 16 cycles of 67M particles with 24 warps 13.15 ms, 28 12.96, 32,
+// with spills, 13.04) owns a contiguous range of tiles, which its warps take in order from a
 // shared-memory counter, so all of them finish within a tile of each other.
-__global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs p) {
+__global__ void __launch_bounds__(896, 1) sweep_smc_pair_kernel(const SweepArgs p) {
   __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
   const uint32_t n_tiles_all = (uint32_t)p.n_tiles;
@@ -228,9 +229,10 @@ __global__ void __launch_bounds__(768, 1) sweep_smc_pair_kernel(const SweepArgs 
 
 // Smart Monte Carlo sweep of the other chain lengths, and of even ones whose
 // tiles would leave more slots empty, in the strips of strip.cuh.  2.1M
-// particles of N = 33: 73.9 us a sweep in tiles, 38.5 us in strips.
+// particles of N = 33: 73.9 us a sweep in tiles, 38.5 us in strips;
+// 20 cycles with 24 warps 799 us, 28 774, 32 838.
 template <typename IDX>
-__global__ void __launch_bounds__(768, 1) sweep_smc_strip_kernel(const SweepArgs p) {
+__global__ void __launch_bounds__(896, 1) sweep_smc_strip_kernel(const SweepArgs p) {
   __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
   const uint32_t chunk = (p.n_items + gridDim.x - 1) / gridDim.x;

@@ -341,8 +341,8 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   } else if (move != 2) {
     // one block per SM: 32 warps in 64 registers without spills for uniform moves
     // (16 cycles of 134M particles with 24 warps 16.56 ms, 28 16.42, 32 16.22; thin
-    // film 2.61, 2.46, 2.43), 24 for smart Monte Carlo's 77 registers
-    s.block = move == 1 ? 768 : 1024;
+    // film 2.61, 2.46, 2.43), 28 for smart Monte Carlo (smc.cu)
+    s.block = move == 1 ? 896 : 1024;
   }
   s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
   s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;

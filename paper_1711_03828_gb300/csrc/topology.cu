@@ -378,7 +378,8 @@ __global__ void __launch_bounds__(256, 3) sweep_topology_kernel(const TopoArgs t
 // positions go to shared memory, where a mover reads its bond partners.  A warp
 // owns G molecules, R lanes each (R: the largest set of any architecture); one
 // block of 28 warps per SM (16 cycles of the stars below with 24 warps 3.18 ms,
-// 28 3.16, 32 and spills 3.49; 24 under smart Monte Carlo) takes its tiles from a
+// 28 3.16, 32 and spills 3.49; three types under smart Monte Carlo 24 1.04, 26 0.95,
+// 28 1.00) takes its tiles from a
 // shared-memory counter; the next tile's positions and the architectures of the
 // one after are loaded ahead.  The moves are those of sweep_topology_kernel, operation for operation.
 // Stars, combs, rings and diblocks of 32 (16.8M particles): 252 us a sweep with
@@ -487,9 +488,9 @@ __device__ __forceinline__ bool topo_move(const TopoArgs& t, TopoSlot& s, const 
 }
 
 template <typename WT, bool MULTI, bool SMC>
-__global__ void __launch_bounds__(SMC ? 768 : 896, 1) sweep_topology_pair_kernel(const TopoArgs t) {
+__global__ void __launch_bounds__(SMC ? 832 : 896, 1) sweep_topology_pair_kernel(const TopoArgs t) {
   __shared__ uint32_t s_next;
-  __shared__ float4 record[SMC ? 24 : 28][TopoTile<false>::REC];
+  __shared__ float4 record[SMC ? 26 : 28][TopoTile<false>::REC];
   const SweepArgs& p = t.s;
   const int lane = threadIdx.x & 31;
   float4* P = record[threadIdx.x >> 5];
@@ -865,7 +866,7 @@ cudaError_t launch_sweep_topology_pair(const TopoArgs& a, int grid, int grid_dty
   void* args[] = {const_cast<TopoArgs*>(&a)};
   return launch_chained(smc ? topology_pair_ptr_of<true>(grid_dtype, types)
                               : topology_pair_ptr_of<false>(grid_dtype, types),
-                          dim3(grid), dim3(smc ? 768 : 896), args, 0, st);
+                          dim3(grid), dim3(smc ? 832 : 896), args, 0, st);
 }
 
 int topology_grid(int grid_dtype, bool big, int sm_count, uint64_t n_tiles, bool types, bool smc) {
