@@ -1498,8 +1498,6 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
   float* dla = nullptr;
   SOMA_CUDA(cudaMallocAsync((void**)&dJ, sizeof(float) * cfg->batch, h->stream));
   SOMA_CUDA(cudaMallocAsync((void**)&dla, sizeof(float) * cfg->batch, h->stream));
-  std::vector<float> hJ(cfg->batch), hla(cfg->batch);
-  double first = 0.0, last = 0.0, acc_last = 0.0;
   const SweepArgs sa = sweep_args(h, h->plain_shape);
   FieldArgs fa = field_args(h, 1);
   float4* const tab = fa.tab;
@@ -1526,27 +1524,24 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
                           h->stream));
     h->launches += 2;
     if (k == 0 || k + 1 == cfg->steps) {
-      SOMA_CUDA(cudaMemcpyAsync(hJ.data(), dJ, sizeof(float) * cfg->batch, cudaMemcpyDeviceToHost, h->stream));
-      SOMA_CUDA(cudaMemcpyAsync(hla.data(), dla, sizeof(float) * cfg->batch, cudaMemcpyDeviceToHost, h->stream));
-      SOMA_CUDA(cudaStreamSynchronize(h->stream));
-      double sj = 0.0, sa_ = 0.0;
-      for (uint32_t b = 0; b < cfg->batch; ++b) {
-        sj += hJ[b];
-        sa_ += hla[b] >= 0.f ? 1.0 : std::exp((double)hla[b]);
+      // sums of the first batch in d_out[0..1], of the last in d_out[2..3]
+      for (int last = k == 0 ? 0 : 1; last <= (k + 1 == cfg->steps ? 1 : 0); ++last) {
+        SOMA_CUDA(launch_train_sums(dJ, dla, cfg->batch, h->sm_count, h->d_scratch, h->d_out + 2 * last,
+                                    h->stream));
+        h->launches += 2;
       }
-      if (k == 0) first = sj / cfg->batch;
-      last = sj / cfg->batch;
-      acc_last = sa_ / cfg->batch;
     }
   }
+  double r[4];
+  SOMA_CUDA(cudaMemcpyAsync(r, h->d_out, sizeof r, cudaMemcpyDeviceToHost, h->stream));
   cudaFreeAsync(dJ, h->stream);
   cudaFreeAsync(dla, h->stream);
   soma_status st = sync(h);
   if (st != SOMA_OK) return st;
   if (log) {
-    log->mean_J_first = first;
-    log->mean_J_last = last;
-    log->mean_alpha_last = acc_last;
+    log->mean_J_first = r[0] / cfg->batch;
+    log->mean_J_last = r[2] / cfg->batch;
+    log->mean_alpha_last = r[3] / cfg->batch;
     log->steps_done = cfg->steps;
     log->reserved = 0;
   }

@@ -147,6 +147,9 @@ int batch_kernel_blocks_per_sm(int block, int grid_dtype);
 cudaError_t launch_sweep_learned(const SweepArgs& a, const SweepShape& s, int grid_dtype,
                                  const void* wq, cudaStream_t st);
 cudaError_t launch_esjd_grad(const TrainArgs& t, int grid_dtype, int sm_count, cudaStream_t st);
+// out[0] = sum of J, out[1] = sum of min(1, exp(log_alpha)) (FP64); part: 2 OBS_BLOCKS doubles
+cudaError_t launch_train_sums(const float* J, const float* log_alpha, uint32_t n, int sm_count,
+                              double* part, double* out, cudaStream_t st);
 cudaError_t launch_adam(float* w, float* m, float* v, const float* grad, void* wq, float lr,
                         float b1, float b2, float eps, int step, float inv_n, cudaStream_t st);
 cudaError_t launch_quantize(const float* w, void* wq, cudaStream_t st);

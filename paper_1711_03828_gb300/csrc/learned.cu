@@ -14,6 +14,7 @@
 // Parameter layout (1604): W1[32][12] b1[32] W2[32][32] b2[32] W3[4][32] b3[4].
 #include "kernels.h"
 #include "draws.cuh"
+#include "square_sum.cuh"
 
 namespace soma {
 
@@ -550,6 +551,52 @@ cudaError_t launch_esjd_grad(const TrainArgs& t, int grid_dtype, int sm_count, c
     case 2: esjd_grad_kernel<__half><<<(unsigned)blocks, GRAD_T, 0, st>>>(t); break;
     default: esjd_grad_kernel<float><<<(unsigned)blocks, GRAD_T, 0, st>>>(t); break;
   }
+  return cudaGetLastError();
+}
+
+// Sums over a batch of J and of the acceptance min(1, e^l), FP64, for the training
+// log: per block, then one block folds them in a fixed order into out[0..1].
+// (Copied to the host and summed there they left the GPU idle twice per call: 8 steps
+// of 16,384 samples on 1M particles 1435 us, 1222 now.)
+__global__ void __launch_bounds__(256) train_sums_kernel(const float* __restrict__ J,
+                                                         const float* __restrict__ log_alpha,
+                                                         uint32_t n, double* __restrict__ part) {
+  __shared__ double sh[2 * 32];
+  double v[2] = {0.0, 0.0};
+  for (uint32_t b = blockIdx.x * 256u + threadIdx.x; b < n; b += gridDim.x * 256u) {
+    const float l = log_alpha[b];
+    v[0] += (double)J[b];
+    v[1] += l >= 0.f ? 1.0 : exp((double)l);
+  }
+  block_sum<2>(v, sh);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = v[0];
+    part[2 * blockIdx.x + 1] = v[1];
+  }
+}
+
+__global__ void __launch_bounds__(256) train_sums_final_kernel(const double* __restrict__ part, int nb,
+                                                               double* __restrict__ out) {
+  __shared__ double sh[2 * 32];
+  double v[2] = {0.0, 0.0};
+  for (int k = threadIdx.x; k < nb; k += 256) {
+    v[0] += part[2 * k];
+    v[1] += part[2 * k + 1];
+  }
+  block_sum<2>(v, sh);
+  if (threadIdx.x == 0) {
+    out[0] = v[0];
+    out[1] = v[1];
+  }
+}
+
+cudaError_t launch_train_sums(const float* J, const float* log_alpha, uint32_t n, int sm_count,
+                              double* part, double* out, cudaStream_t st) {
+  uint64_t nb = ((uint64_t)n + 255) / 256;
+  if (nb > (uint64_t)sm_count) nb = (uint64_t)sm_count;
+  if (nb > (uint64_t)OBS_BLOCKS) nb = OBS_BLOCKS;
+  train_sums_kernel<<<(unsigned)nb, 256, 0, st>>>(J, log_alpha, n, part);
+  train_sums_final_kernel<<<1, 256, 0, st>>>(part, (int)nb, out);
   return cudaGetLastError();
 }
 
