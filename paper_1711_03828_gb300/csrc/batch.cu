@@ -6,7 +6,7 @@
 // sizes, chain lengths, compositions, chiN, replicas of one seed) shares a
 // single persistent launch: the tiles of all systems are cut into work items
 // of contiguous tiles of one system; block j takes items j, j + grid, ... and
-// its warps walk an item's tiles with the same tile body as the single-system
+// its warps take the items' tiles in turn with the same tile body as the single-system
 // kernel (pair_body.cuh), so every system evolves bit-identically to the same
 // system run alone.  The host lays the items out either as fixed-length items
 // of each system in turn or as one equal contiguous range of the concatenated
@@ -19,73 +19,121 @@
 
 namespace soma {
 
+// A block's warps take the tiles of its items from a shared counter, so that they
+// end within a tile of each other.  The constants of the system a warp works on
+// (and of the next tile's, when it is another) lie in shared memory, those of the
+// cell fold in registers as well: 80 registers without spills at 24 warps an SM.
+// With all of them in registers the kernel spilled, and waited for its blocks'
+// slowest warps; with none it takes 71 but more loads a tile.  Cycles of 64 systems,
+// 40M particles in all, spilled and dealt in turn: 393 us (373 with 16 warps), none in
+// registers 381, with 32 warps 377, as here 379; 16 systems of 10.6M in all: 125 (110),
+// 106, 105, 105.  One list of tiles for all blocks of an SM through a counter in
+// global memory was slower (385, 144): the blocks that share one do not share an SM,
+// and their gathers do not repeat in one L1.
 template <typename WT>
 __global__ void __launch_bounds__(256, 3) sweep_batch_kernel(const BatchArgs p) {
+  __shared__ BatchSys s_sys[8][2];
+  __shared__ uint32_t s_id[8][2];   // the systems in s_sys
+  __shared__ uint32_t s_next;
   const int lane = threadIdx.x & 31;
-  const uint32_t warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const uint32_t warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_next = 0u;
+  __syncthreads();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
   const bool odd = ((s64 + 1ull) & 1ull) != 0;
 
-  uint32_t cur = 0xFFFFFFFFu;
-  BatchSys S;
-  PairLane<WT> L;
-  uint32_t* nacc = nullptr;
-  uint32_t ctr3 = 0, TN = 0;
-  unsigned my_acc = 0;
-
-  for (uint32_t item = blockIdx.x; item < p.n_items; item += gridDim.x) {
-    const BatchItem it = p.items[item];
-    if (it.sys != cur) {
-      if (cur != 0xFFFFFFFFu) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
-        if (lane == 0 && my_acc) atomicAdd(S.counters + 1, (unsigned long long)my_acc);
-        my_acc = 0;
+  // the walk over the block's items: the item of the tile claimed last, the
+  // block's tiles up to its end, its first tile less the tiles before it, the
+  // slot of its system's constants
+  uint32_t item = blockIdx.x - gridDim.x, end = 0, shift = 0, tile = 0;
+  int slot = 0;
+  if (lane < 2) s_id[warp][lane] = 0xFFFFFFFFu;
+  auto claim = [&]() -> bool {
+    uint32_t u = 0u;
+    if (lane == 0) u = atomicAdd(&s_next, 1u);
+    u = __shfl_sync(FULL, u, 0);
+    if (u >= end) {
+      uint32_t sys;
+      do {
+        item += gridDim.x;
+        if (item >= p.n_items) {
+          item -= gridDim.x;
+          return false;
+        }
+        const BatchItem it = p.items[item];
+        shift = it.t0 - end;
+        end += it.t1 - it.t0;
+        sys = it.sys;
+      } while (u >= end);
+      __syncwarp();
+      if (sys != s_id[warp][slot]) {   // the other slot: the tile claimed before has yet to be swept
+        slot ^= 1;
+        __syncwarp();
+        const uint32_t* from = reinterpret_cast<const uint32_t*>(p.sys + sys);
+        uint32_t* to = reinterpret_cast<uint32_t*>(&s_sys[warp][slot]);
+        for (uint32_t k = lane; k < sizeof(BatchSys) / 4u; k += 32u) to[k] = from[k];
+        if (lane == 0) s_id[warp][slot] = sys;
+        __syncwarp();
       }
-      cur = it.sys;
-      S = p.sys[cur];
-      L.init(lane, S.g.N, S.g.N_A, S.wA, S.wB);
-      nacc = odd ? S.n1 : S.n0;
-      ctr3 = (PURPOSE_MOVE << 24) | (S.g.replica & 0xFFFFFFu);
-      TN = S.G * S.g.N;
     }
-    auto lane_ok = [&](uint32_t t) { return L.in_tile(t < S.full_tiles, S.last_rows); };
-    const uint32_t dense_tiles = TN == 64u ? S.full_tiles : 0u;   // no masks needed
-    const uint32_t t0 = it.t0 + warp;
-    float2 px = make_float2(0.f, 0.f), py = px, pz = px;
-    if (t0 < it.t1 && lane_ok(t0)) {
-      const uint32_t b0 = t0 * TN + L.li0;
+    tile = u + shift;
+    return true;
+  };
+  float2 px = make_float2(0.f, 0.f), py = px, pz = px;
+  auto load = [&]() {   // the claimed tile's positions
+    const BatchSys& S = s_sys[warp][slot];
+    const uint32_t rows = tile < S.full_tiles ? S.G * S.g.N : S.last_rows;
+    if (2u * (uint32_t)lane < rows) {
+      const uint32_t b0 = tile * (S.G * S.g.N) + 2u * (uint32_t)lane;
       px = __ldcs(reinterpret_cast<const float2*>(S.x + b0));
       py = __ldcs(reinterpret_cast<const float2*>(S.y + b0));
       pz = __ldcs(reinterpret_cast<const float2*>(S.z + b0));
     }
-    for (uint32_t tile = t0; tile < it.t1; tile += nwarps) {
-      const bool valid = lane_ok(tile);
-      const uint32_t base = tile * TN + L.li0;
-      const float x0 = px.x, x1 = px.y, y0 = py.x, y1 = py.y, z0 = pz.x, z1 = pz.y;
-      const uint32_t nt = tile + nwarps;
-      if (nt < it.t1 && lane_ok(nt)) {
-        const uint32_t bn = nt * TN + L.li0;
-        px = __ldcs(reinterpret_cast<const float2*>(S.x + bn));
-        py = __ldcs(reinterpret_cast<const float2*>(S.y + bn));
-        pz = __ldcs(reinterpret_cast<const float2*>(S.z + bn));
-      }
-      if (tile < dense_tiles)
-        my_acc += pair_tile<WT, uint32_t, false, false>(S.g, p.keys, L, S.x, S.y, S.z, nacc, base, base,
-                                                 true, sweep, ctr3, S.set_order_random, S.a, S.K_b, x0,
-                                                 x1, y0, y1, z0, z1);
-      else
-        my_acc += pair_tile<WT, uint32_t, true, false>(S.g, p.keys, L, S.x, S.y, S.z, nacc, base, base,
-                                                valid, sweep, ctr3, S.set_order_random, S.a, S.K_b, x0,
-                                                x1, y0, y1, z0, z1);
-    }
-  }
-  if (cur != 0xFFFFFFFFu) {
+  };
+  auto flush = [&](uint32_t k, unsigned n) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) my_acc += __shfl_xor_sync(FULL, my_acc, o);
-    if (lane == 0 && my_acc) atomicAdd(S.counters + 1, (unsigned long long)my_acc);
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
+    if (lane == 0 && n) atomicAdd(p.sys[k].counters + 1, (unsigned long long)n);
+  };
+
+  PairLane<WT> L;
+  Geom g = {};
+  float a = 0.f, K_b = 0.f;
+  int at = -1;   // the slot of the system L belongs to
+  unsigned my_acc = 0;
+  bool have = claim();
+  if (have) load();
+  while (have) {
+    const BatchSys& S = s_sys[warp][slot];
+    if (slot != at) {
+      if (at >= 0) flush(s_id[warp][at], my_acc);
+      my_acc = 0;
+      at = slot;
+      g = S.g;
+      a = S.a;
+      K_b = S.K_b;
+      L.init(lane, S.g.N, S.g.N_A, S.wA, S.wB);
+    }
+    const uint32_t t = tile;
+    const float x0 = px.x, x1 = px.y, y0 = py.x, y1 = py.y, z0 = pz.x, z1 = pz.y;
+    have = claim();
+    if (have) load();
+    uint32_t* nacc = odd ? S.n1 : S.n0;
+    __builtin_assume(__isGlobal(nacc));
+    const uint32_t ctr3 = (PURPOSE_MOVE << 24) | (g.replica & 0xFFFFFFu);
+    const bool full = t < S.full_tiles;
+    const uint32_t base = t * L.tile_rows + L.li0;
+    if (full && L.tile_rows == 64u)   // no masks needed
+      my_acc += pair_tile<WT, uint32_t, false, false>(g, p.keys, L, S.x, S.y, S.z, nacc, base, base,
+                                               true, sweep, ctr3, S.set_order_random, a, K_b, x0,
+                                               x1, y0, y1, z0, z1);
+    else
+      my_acc += pair_tile<WT, uint32_t, true, false>(g, p.keys, L, S.x, S.y, S.z, nacc, base, base,
+                                              L.in_tile(full, S.last_rows), sweep, ctr3,
+                                              S.set_order_random, a, K_b, x0, x1, y0, y1, z0, z1);
   }
+  if (at >= 0) flush(s_id[warp][at], my_acc);
 }
 
 // Field update of every system: one thread per cell of the concatenated grids;
