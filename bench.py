@@ -290,7 +290,8 @@ def measured_traffic(workload_name):
 def sweep_kernel_name(d, architectures=False):
     """The sweep kernel libsoma launches for this description."""
     if architectures:
-        return "sweep_molecule_topology_kernel" if d.set_order == 2 else "sweep_topology_kernel"
+        # the workloads' molecules (stars, combs, even rings, chains of 32) have two sets
+        return "sweep_molecule_topology_kernel" if d.set_order == 2 else "sweep_topology_pair_kernel"
     pair = d.N % 2 == 0 and d.N <= 64
     if d.move == 1:
         fills = pair and (64 // d.N) * (d.N // 2 + 1) >= 32   # tiles fill the lanes as strips do

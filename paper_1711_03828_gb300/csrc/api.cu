@@ -405,6 +405,7 @@ TypesArgs types_args(soma_t* h, int after_sweep) {
   a.n0 = h->nt[0];
   a.n1 = h->nt[1];
   a.w = h->wt;
+  a.tab = h->d_smc;
   a.d_sweep = h->d_counters;
   a.n_types = h->n_types;
   a.after_sweep = after_sweep;
@@ -419,16 +420,11 @@ TypesArgs types_args(soma_t* h, int after_sweep) {
   return a;
 }
 
-// the field update of one cycle: the packed A | B grid (with the table of a smart
-// Monte Carlo system) or the type planes and their table
+// the field update of one cycle (with the table of a smart Monte Carlo system): the
+// packed A | B grid or the type planes
 cudaError_t launch_fields_any(soma_t* h, const FieldArgs& fa, const TypesArgs& ta) {
   if (!h->n_types) return launch_fields(fa, h->d_err + 1, h->grid_dtype, h->sm_count, h->stream);
-  cudaError_t e = launch_fields_types(ta, h->d_err + 1, h->sm_count, h->stream);
-  if (e == cudaSuccess && h->d_smc) {
-    ++h->launches;
-    e = launch_smc_table_planes(h->g, h->wt, h->n_types, h->d_smc, h->sm_count, h->stream);
-  }
-  return e;
+  return launch_fields_types(ta, h->d_err + 1, h->sm_count, h->stream);
 }
 
 cudaError_t launch_sweep_any(soma_t* h, const SweepArgs& sa) {

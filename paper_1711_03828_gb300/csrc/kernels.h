@@ -165,11 +165,6 @@ const void* molecule_kernel(uint64_t n_chains, uint32_t N, int grid_dtype, int s
 int molecule_grid(uint64_t n_chains, uint32_t N, int grid_dtype, int sm_count);
 // smart Monte Carlo sweep kernel: pair tiles or strips (big: 64-bit indices)
 const void* smc_kernel_ptr(bool strip, bool big);
-// Smart Monte Carlo table for n_t types (omega and the central-difference field
-// force per cell, one float4 plane per type) from the FP32 planes w, rebuilt after
-// every field update; two types have theirs from the field kernel
-cudaError_t launch_smc_table_planes(const Geom& g, const float* w, uint32_t planes, float4* tab,
-                                    int sm_count, cudaStream_t st);
 
 // Molecules of any architecture (topology.cu): the architecture array of
 // Sec. 3.2.1 and the independent sets derived from it.
@@ -249,6 +244,7 @@ struct TypesArgs {
   uint32_t* n0;              // count planes, n_types * cells each; the sweep of step s
   uint32_t* n1;              // counts into planes (s+1)&1
   float* w;                  // field planes, n_types * cells
+  float4* tab;               // table of a smart Monte Carlo sweep, n_types * cells (or NULL)
   unsigned long long* d_sweep;
   uint32_t n_types;
   int after_sweep;           // as FieldArgs

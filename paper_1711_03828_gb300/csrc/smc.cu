@@ -20,45 +20,6 @@
 
 namespace soma {
 
-// omega at the cell and minus its central-difference gradient (the field force).
-template <typename WT>
-__device__ __forceinline__ float field_and_force(const Geom& g, const WT* w, uint32_t cx, uint32_t cy,
-                                                 uint32_t cz, float& fx, float& fy, float& fz) {
-  const uint32_t nx = g.nx, ny = g.ny, nz = g.nz;
-  const uint32_t row = (cz * ny + cy) * nx;
-  const uint32_t xm = cx == 0 ? nx - 1 : cx - 1, xp = cx + 1 == nx ? 0 : cx + 1;
-  const uint32_t ym = cy == 0 ? ny - 1 : cy - 1, yp = cy + 1 == ny ? 0 : cy + 1;
-  const uint32_t zm = cz == 0 ? nz - 1 : cz - 1, zp = cz + 1 == nz ? 0 : cz + 1;
-  fx = -0.5f * (load_w<WT>(w, row + xp) - load_w<WT>(w, row + xm));
-  fy = -0.5f * (load_w<WT>(w, (cz * ny + yp) * nx + cx) - load_w<WT>(w, (cz * ny + ym) * nx + cx));
-  fz = -0.5f * (load_w<WT>(w, (zp * ny + cy) * nx + cx) - load_w<WT>(w, (zm * ny + cy) * nx + cx));
-  return load_w<WT>(w, row + cx);
-}
-
-// The table of a smart Monte Carlo sweep for n_t types (of two types: made by the
-// field kernel): one plane of float4 per type, omega and the field force, from
-// the FP32 field planes w (n_types * cells).
-__global__ void smc_table_planes_kernel(const Geom g, const float* __restrict__ w, uint32_t planes,
-                                        float4* __restrict__ tab) {
-  chained_begin();
-  const uint32_t nx = g.nx, ny = g.ny;
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < g.cells;
-       c += gridDim.x * blockDim.x) {
-    const uint32_t cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
-    for (uint32_t t = 0; t < planes; ++t) {
-      float fx, fy, fz;
-      const float v = field_and_force<float>(g, w + (size_t)t * g.cells, cx, cy, cz, fx, fy, fz);
-      tab[(size_t)t * g.cells + c] = make_float4(v, fx, fy, fz);
-    }
-  }
-}
-
-cudaError_t launch_smc_table_planes(const Geom& g, const float* w, uint32_t planes, float4* tab,
-                                    int sm_count, cudaStream_t st) {
-  void* args[] = {const_cast<Geom*>(&g), &w, &planes, &tab};
-  return launch_chained((const void*)smc_table_planes_kernel, dim3(4 * sm_count), dim3(256), args, 0, st);
-}
-
 // ---------------------------------------------------------------------------
 // Smart Monte Carlo step for even N <= 64 in the paired layout of
 // pair_body.cuh: lane l holds the even particle 2l and the odd particle 2l+1

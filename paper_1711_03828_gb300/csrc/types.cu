@@ -19,41 +19,76 @@ namespace soma {
 
 namespace {
 
+// omega of every type in a cell, from the count planes n.
+template <uint32_t T>
+__device__ __forceinline__ void omega_types(const TypesArgs& p, const uint32_t* __restrict__ n, uint32_t c,
+                                            float (&w)[T]) {
+  float phi[T];
+  float total = 0.f;
+#pragma unroll
+  for (uint32_t t = 0; t < T; ++t) {
+    phi[t] = (float)n[(size_t)t * p.g.cells + c] * p.inv_rho;
+    total += phi[t];
+  }
+  const float comp = p.kappa0 * (total - 1.f);
+#pragma unroll
+  for (uint32_t i = 0; i < T; ++i) {
+    float v = comp;
+#pragma unroll
+    for (uint32_t k = 0; k < T; ++k) {
+      if (k == i) continue;
+      const float chi0 = p.chi0[i * TYPES_MAX + k];
+      v = p.hamiltonian ? fmaf(chi0, phi[k], v) : fmaf(-0.5f * chi0, phi[i] - phi[k], v);
+    }
+    w[i] = v;
+  }
+}
+
 // One thread per cell: reads the planes being read, clears the planes the
 // next sweep counts into, writes every type's field; after a sweep the last
 // block to finish advances the device sweep counter (as fields_kernel does).
+// TAB: the table of a smart Monte Carlo sweep in the same pass, per type and cell
+// omega and minus its central difference along each axis, the neighbours' omega
+// from their counts.  Three types, 2.1M particles, 20 cycles: with a second kernel
+// that read the planes again 956 us, so 939 (with the number of types a run-time
+// bound 979: the unused types' guards cost more than the launch).
+template <uint32_t T, bool TAB>
 __global__ void __launch_bounds__(256) fields_types_kernel(const TypesArgs p, unsigned* arrive) {
   chained_begin();
   const unsigned long long s = *p.d_sweep;
   const int rd = p.after_sweep ? (int)((s + 1ull) & 1ull) : (int)(s & 1ull);
   const uint32_t* __restrict__ nr = rd ? p.n1 : p.n0;
   uint32_t* __restrict__ nc = rd ? p.n0 : p.n1;
-  const uint32_t cells = p.g.cells, T = p.n_types;
+  const uint32_t cells = p.g.cells;
+  const uint32_t nx = p.g.nx, ny = p.g.ny, nz = p.g.nz;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += stride) {
-    float phi[TYPES_MAX];
-    float total = 0.f;
+    float w[T];
+    omega_types(p, nr, c, w);
 #pragma unroll
-    for (uint32_t t = 0; t < TYPES_MAX; ++t) {
-      phi[t] = 0.f;
-      if (t < T) {
-        phi[t] = (float)nr[(size_t)t * cells + c] * p.inv_rho;
-        nc[(size_t)t * cells + c] = 0u;
-        total += phi[t];
-      }
+    for (uint32_t t = 0; t < T; ++t) {
+      nc[(size_t)t * cells + c] = 0u;
+      p.w[(size_t)t * cells + c] = w[t];
     }
-    const float comp = p.kappa0 * (total - 1.f);
+    if (TAB) {
+      const uint32_t cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
+      const uint32_t lo[3] = {cx == 0 ? c + nx - 1 : c - 1, cy == 0 ? c + (ny - 1) * nx : c - nx,
+                              cz == 0 ? c + (nz - 1) * ny * nx : c - ny * nx};
+      const uint32_t hi[3] = {cx + 1 == nx ? c + 1 - nx : c + 1,
+                              cy + 1 == ny ? c - (ny - 1) * nx : c + nx,
+                              cz + 1 == nz ? c - (nz - 1) * ny * nx : c + ny * nx};
+      float f[3][T];
 #pragma unroll
-    for (uint32_t i = 0; i < TYPES_MAX; ++i) {
-      if (i >= T) break;
-      float v = comp;
+      for (int d = 0; d < 3; ++d) {
+        float wl[T], wh[T];
+        omega_types(p, nr, lo[d], wl);
+        omega_types(p, nr, hi[d], wh);
 #pragma unroll
-      for (uint32_t k = 0; k < TYPES_MAX; ++k) {
-        if (k >= T || k == i) continue;
-        const float chi0 = p.chi0[i * TYPES_MAX + k];
-        v = p.hamiltonian ? fmaf(chi0, phi[k], v) : fmaf(-0.5f * chi0, phi[i] - phi[k], v);
+        for (uint32_t t = 0; t < T; ++t) f[d][t] = -0.5f * (wh[t] - wl[t]);
       }
-      p.w[(size_t)i * cells + c] = v;
+#pragma unroll
+      for (uint32_t t = 0; t < T; ++t)
+        p.tab[(size_t)t * cells + c] = make_float4(w[t], f[0][t], f[1][t], f[2][t]);
     }
   }
   if (p.after_sweep) {
@@ -180,6 +215,19 @@ cudaError_t launch_pack_type_pair(const uint32_t* n, uint32_t cells, uint32_t ti
   return cudaGetLastError();
 }
 
+template <bool TAB>
+static const void* fields_types_ptr(uint32_t n_types) {
+  switch (n_types) {
+    case 2: return (const void*)fields_types_kernel<2, TAB>;
+    case 3: return (const void*)fields_types_kernel<3, TAB>;
+    case 4: return (const void*)fields_types_kernel<4, TAB>;
+    case 5: return (const void*)fields_types_kernel<5, TAB>;
+    case 6: return (const void*)fields_types_kernel<6, TAB>;
+    case 7: return (const void*)fields_types_kernel<7, TAB>;
+    default: return (const void*)fields_types_kernel<8, TAB>;
+  }
+}
+
 cudaError_t launch_fields_types(const TypesArgs& a, unsigned* arrive, int sm_count,
                                 cudaStream_t st) {
   uint64_t blocks = ((uint64_t)a.g.cells + 255) / 256;
@@ -187,7 +235,8 @@ cudaError_t launch_fields_types(const TypesArgs& a, unsigned* arrive, int sm_cou
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   void* args[] = {const_cast<TypesArgs*>(&a), &arrive};
-  return launch_chained((const void*)fields_types_kernel, dim3((unsigned)blocks), dim3(256), args, 0, st);
+  const void* fn = a.tab ? fields_types_ptr<true>(a.n_types) : fields_types_ptr<false>(a.n_types);
+  return launch_chained(fn, dim3((unsigned)blocks), dim3(256), args, 0, st);
 }
 
 cudaError_t launch_histogram_types(const Geom& g, const float* x, const float* y, const float* z,
