@@ -92,7 +92,7 @@ struct soma_t {
   float* pos = nullptr;
   uint32_t* n[2] = {nullptr, nullptr};
   uint32_t* n_spare = nullptr;               // third count buffer of a resident system
-  ResidentShape resident{0, 0, 0};              // many cycles per launch (resident.cu)
+  ResidentShape resident{0, 0, 0, 0};           // many cycles per launch (resident.cu)
   void* w[2] = {nullptr, nullptr};
   unsigned long long* d_counters = nullptr;  // [0] sweep, [1] accepted
   unsigned* d_err = nullptr;                 // [0] error bits, [1] arrival counter,
@@ -656,7 +656,7 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
   // a small system under uniform moves of linear chains: one launch for up to
   // RESIDENT_CYCLES cycles (per-kernel timing needs the two kernels)
   if (h->resident.grid && !h->timing && !h->has_topo && !h->n_types) {
-    for (; done < n;) {
+    while (n - done >= h->resident.min_cycles) {
       ResidentArgs a;
       a.s = sweep_args(h, h->shape);
       a.f = field_args(h, 1);
@@ -672,16 +672,15 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
       h->host_sweep += a.cycles;
       done += a.cycles;
     }
-    return SOMA_OK;
   }
-  if (!h->timing && n >= GRAPH_CHUNK) {
+  if (!h->timing && n - done >= GRAPH_CHUNK) {
     if (!h->graph) {
       soma_status st = build_graph(h);
       if (st != SOMA_OK) return st;
     }
     while (n - done >= GRAPH_CHUNK) {
       SOMA_CUDA(cudaGraphLaunch(h->graph, h->stream));
-      h->launches += (h->d_smc && h->n_types ? 3 : 2) * GRAPH_CHUNK;
+      h->launches += 2 * GRAPH_CHUNK;
       h->t.sweep_launches += GRAPH_CHUNK;
       h->t.field_launches += GRAPH_CHUNK;
       h->host_sweep += GRAPH_CHUNK;

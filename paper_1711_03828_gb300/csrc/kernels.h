@@ -62,6 +62,7 @@ cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int gr
 struct ResidentShape {
   int grid, block;
   size_t cluster_smem;   // shared memory of the one-cluster kernel (0: the cooperative one)
+  uint32_t min_cycles;   // shorter calls take the two kernels
 };
 struct ResidentArgs {
   SweepArgs s;
@@ -71,10 +72,17 @@ struct ResidentArgs {
   unsigned* arrive;    // blocks that have ended, 0 between launches
   uint32_t cycles;
 };
-// Largest system of the resident sweep, in tiles of 64 slots per SM: three rounds of
-// 32 warps.  Resident against two kernels a cycle: 27 tiles per SM 7.1 and 9.5 us, 40
-// 8.7 and 11.9, 61 11.4 and 12.1, 91 13.8 and 14.1, 121 16.8 and 16.6, 162 19.3 and 19.2.
-constexpr uint64_t RESIDENT_TILES_PER_SM = 96;
+// Largest system of the resident sweep, in tiles of 64 slots per SM: two rounds of
+// 32 warps.  Resident against two kernels a cycle in long calls: 27 tiles per SM 7.4
+// and 9.3 us, 40 9.1 and 11.1, 61 11.0 and 11.9, 91 14.1 and 14.5 (16 cycles 234 and
+// 229), 121 16.8 and 16.6.
+constexpr uint64_t RESIDENT_TILES_PER_SM = 64;
+// Fewest cycles of a call that take it: two, and one more per 16 tiles per SM.  Its
+// launch and last field update cost what some cycles gain; calls back to back,
+// resident against two kernels: one cycle at 3 tiles per SM 9.9 and 7.2 us, 40 16.3
+// and 11.5; two at 8 14.6 and 14.8, 27 22.8 and 19.0; four at 40 42.6 and 45.3, 61 49.3
+// and 47.4; eight at 61 90.6 and 95.0.
+constexpr uint64_t RESIDENT_TILES_PER_CYCLE = 16;
 // One cluster: 16 blocks of up to 16 warps, a tile each, and the counts three times
 // in a block's shared memory (96 KB at the limit).  With 32 warps on its 16 SMs
 // their issue slots are the time: 32,768 particles 4.4 us a cycle against 4.2 over

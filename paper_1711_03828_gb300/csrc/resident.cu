@@ -13,7 +13,7 @@
 // followed by the field update and leaves the buffers as the two-kernel cycle
 // does (n[s&1] current, the other cleared, the third cleared).  Per cycle, against
 // the two kernels under a CUDA graph: 4,096 particles 6.6 -> 3.4 us, 32,768 7.1 ->
-// 4.2, 262,144 9.5 -> 7.1, 393,216 11.9 -> 8.7, 884,736 14.1 -> 13.8.
+// 4.2, 262,144 9.5 -> 7.1, 393,216 11.9 -> 8.7, 589,824 11.9 -> 11.0.
 //
 // Systems of at most one tile per warp of one cluster of 16 blocks
 // (resident_cluster_kernel) never leave the chip between cycles: positions stay
@@ -348,12 +348,12 @@ static bool cluster_shape(uint64_t n_tiles, uint32_t cells, int grid_dtype, Resi
       return false;
     }
   }
-  *r = ResidentShape{CLUSTER_BLOCKS, 32 * warps, smem};
+  *r = ResidentShape{CLUSTER_BLOCKS, 32 * warps, smem, 2};
   return true;
 }
 
 ResidentShape resident_shape(const SweepShape& s, uint32_t cells, int grid_dtype, int sm_count) {
-  ResidentShape r{0, 0, 0};
+  ResidentShape r{0, 0, 0, 0};
   int dev = 0, coop = 0;
   if (s.move != 0 || !s.pair || s.strip || s.big || s.molecule) return r;
   if (s.n_tiles > (uint64_t)sm_count * RESIDENT_TILES_PER_SM) return r;
@@ -366,6 +366,7 @@ ResidentShape resident_shape(const SweepShape& s, uint32_t cells, int grid_dtype
   const uint64_t per = (s.n_tiles + (uint64_t)r.grid - 1) / (uint64_t)r.grid;
   const uint64_t rounds = (per + 31) / 32;
   r.block = 32 * (int)((per + rounds - 1) / rounds);
+  r.min_cycles = 2u + (uint32_t)(s.n_tiles / (RESIDENT_TILES_PER_CYCLE * (uint64_t)sm_count));
   return r;
 }
 
