@@ -93,6 +93,10 @@ struct soma_t {
   uint32_t* n[2] = {nullptr, nullptr};
   uint32_t* n_spare = nullptr;               // third count buffer of a resident system
   ResidentShape resident{0, 0, 0, 0};           // many cycles per launch (resident.cu)
+  // The planes w are not what the counts give with the external fields and the
+  // density as they are now: a change of those takes effect at the next field
+  // update, so until then a sweep has to read the planes.
+  bool fields_behind = false;
   void* w[2] = {nullptr, nullptr};
   unsigned long long* d_counters = nullptr;  // [0] sweep, [1] accepted
   unsigned* d_err = nullptr;                 // [0] error bits, [1] arrival counter,
@@ -451,6 +455,7 @@ soma_status one_cycle(soma_t* h) {
   const TypesArgs ta = types_args(h, 1);
   st = timed(h, 1, [&] { return launch_fields_any(h, fa, ta); });
   if (st != SOMA_OK) return st;
+  if (!h->n_types) h->fields_behind = false;
   ++h->host_sweep;
   return SOMA_OK;
 }
@@ -507,6 +512,7 @@ soma_status update_fields(soma_t* h) {
   ++h->launches;
   SOMA_CUDA(launch_fields_any(h, field_args(h, 0), types_args(h, 0)));
   ++h->launches;
+  h->fields_behind = false;
   return SOMA_OK;
 }
 
@@ -656,6 +662,12 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
   // a small system under uniform moves of linear chains: one launch for up to
   // RESIDENT_CYCLES cycles (per-kernel timing needs the two kernels)
   if (h->resident.grid && !h->timing && !h->has_topo && !h->n_types) {
+    // it evaluates the fields of its first cycle too, instead of reading the planes
+    if (h->fields_behind && n > 0) {
+      soma_status st = one_cycle(h);
+      if (st != SOMA_OK) return st;
+      done = 1;
+    }
     while (n - done >= h->resident.min_cycles) {
       ResidentArgs a;
       a.s = sweep_args(h, h->shape);
@@ -680,6 +692,7 @@ soma_status soma_sweep(soma_t* h, uint32_t n) {
     }
     while (n - done >= GRAPH_CHUNK) {
       SOMA_CUDA(cudaGraphLaunch(h->graph, h->stream));
+      if (!h->n_types) h->fields_behind = false;
       h->launches += 2 * GRAPH_CHUNK;
       h->t.sweep_launches += GRAPH_CHUNK;
       h->t.field_launches += GRAPH_CHUNK;
@@ -868,6 +881,7 @@ soma_status soma_set_external(soma_t* h, const float* ext, const uint8_t* forbid
   const size_t cells = h->g.cells;
   const cudaMemcpyKind k = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   cudaError_t e;
+  h->fields_behind = true;
   if (ext) {
     if (!h->d_ext) {
       e = cudaMalloc((void**)&h->d_ext, sizeof(float) * 2 * cells);
@@ -899,6 +913,7 @@ void restore_particles(soma_t* h) {
   h->rho_cell = tmp.rho_cell;
   h->g.particles = tmp.g.particles;
   h->M_real = h->M;
+  h->fields_behind = true;
 }
 }  // namespace
 
@@ -1058,6 +1073,7 @@ soma_status soma_set_topology(soma_t* h, const uint32_t* words, uint64_t n_words
   if (!h->desc.n_chains_total) {
     h->g.particles = present;
     h->rho_cell = (double)present / (double)h->g.cells;
+    h->fields_behind = true;
   }
   h->topo_R = pairs.R;
   h->topo_G = pairs.G;

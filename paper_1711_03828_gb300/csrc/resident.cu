@@ -23,6 +23,10 @@
 // shared-memory accesses and the two meetings of a cycle hardware cluster
 // barriers: 4,096 particles 3.4 -> 2.1 us a cycle, 13,664 3.9 -> 2.9.
 //
+// The planes w are written, not read: a handle whose planes do not follow from the
+// counts with its external fields and density as they are (they were changed since
+// the last field update) runs a cycle of the two kernels first.
+//
 // The larger launch is cooperative (the blocks wait on one another, so all must be
 // resident: one block per SM at most).  A wait gives up after 2^26 polls, sets
 // the sticky timeout bit and ends the kernel.
