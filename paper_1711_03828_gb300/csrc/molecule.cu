@@ -238,14 +238,24 @@ __global__ void __launch_bounds__(MOL_BLOCK, 8) sweep_molecule_topology_kernel(c
 // on an SM at one lane each (67M particles of N = 64: 1627, 1506 / 1070 / 1173 us);
 // else one (134M of N = 32: 1984, 1871 / 2612 / 2424 us). The line: 67M
 // particles of N = 40, 1111 / 1159 us; of N = 48, 1187 / 1145.
+constexpr uint32_t MOL_ONE_LANE_N = 44;   // longest chains of one lane
+constexpr uint32_t MOL_N = 256;           // longest chains
 uint32_t molecule_lanes(uint64_t n_chains, uint32_t N, int sm_count) {
   if (n_chains < (uint64_t)sm_count * 4u * 32u) return 4u;
-  return N > 44u ? 2u : 1u;
+  return N > MOL_ONE_LANE_N ? 2u : 1u;
 }
 
 // shared memory of a block for chains of N
 static size_t molecule_smem(uint32_t N, uint32_t lanes) {
   return (size_t)3 * MOL_BLOCK / lanes * N * sizeof(float);
+}
+
+// Allows a kernel the shared memory of the longest chains it is ever launched for,
+// whichever system asks: the limit belongs to the kernel, and one set to a system's
+// own chains refuses the launches of the longer ones created before it.
+static cudaError_t molecule_allow_smem(const void* fn, uint32_t lanes) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)molecule_smem(lanes == 1u ? MOL_ONE_LANE_N : MOL_N, lanes));
 }
 
 template <uint32_t LANES>
@@ -271,8 +281,10 @@ static const void* molecule_ptr_of(int grid_dtype) {
                            : (const void*)sweep_molecule_kernel<float, LANES>;
 }
 
-// Blocks of a launch: every group of chains its own warp, up to what fits.
+// Blocks of a launch: every group of chains its own warp, up to what fits (0, which
+// the launch refuses, if the kernel cannot have its shared memory).
 static int molecule_blocks(const void* fn, size_t smem, int sm_count, uint64_t n_chains, uint32_t lanes) {
+  if (molecule_allow_smem(fn, lanes) != cudaSuccess) return 0;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, MOL_BLOCK, smem);
   if (per_sm < 1) per_sm = 1;
@@ -285,10 +297,7 @@ static int molecule_blocks(const void* fn, size_t smem, int sm_count, uint64_t n
 int molecule_topology_grid(uint32_t N, int grid_dtype, int sm_count, uint64_t n_chains, bool types) {
   const uint32_t lanes = molecule_lanes(n_chains, N, sm_count);
   const void* fn = molecule_topology_ptr(grid_dtype, types, lanes);
-  const size_t smem = molecule_smem(N, lanes);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return molecule_blocks(fn, smem, sm_count, n_chains, lanes);
+  return molecule_blocks(fn, molecule_smem(N, lanes), sm_count, n_chains, lanes);
 }
 
 cudaError_t launch_molecule_topology(const TopoArgs& a, int grid, int grid_dtype, int sm_count,
@@ -310,8 +319,6 @@ const void* molecule_kernel(uint64_t n_chains, uint32_t N, int grid_dtype, int s
 int molecule_grid(uint64_t n_chains, uint32_t N, int grid_dtype, int sm_count) {
   size_t smem = 0;
   const void* fn = molecule_kernel(n_chains, N, grid_dtype, sm_count, &smem);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   return molecule_blocks(fn, smem, sm_count, n_chains, molecule_lanes(n_chains, N, sm_count));
 }
 
