@@ -12,6 +12,8 @@
 //   scratch     FP64 partial sums of the observables and S(q) reductions.
 // A cycle is two launches (sweep, fields); soma_sweep replays them from a
 // CUDA graph of GRAPH_CHUNK cycles when timing is off.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -826,16 +828,36 @@ soma_status soma_get_positions(soma_t* h, float* dst, size_t n, int dst_on_devic
 }
 
 namespace {
-// Device memory of the current device (a kernel may read it); managed memory,
-// another device's and anything unknown go through a copy call.
-bool on_this_device(const void* p) {
+// Whether a kernel may read n floats at p: device memory of the current device,
+// on a 4-byte boundary, all of it in one allocation.  Anything else (managed memory,
+// another device's, a range that the copy calls check and refuse) goes through a
+// copy call.
+bool readable_floats(const float* p, size_t n) {
+  typedef CUresult (*RangeFn)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const RangeFn range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &found) !=
+            cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      f = nullptr;
+    }
+    return (RangeFn)f;
+  }();
+  const uintptr_t at = (uintptr_t)p;
   cudaPointerAttributes a;
   int dev = -1;
+  if (!range || at % sizeof(float) != 0) return false;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     (void)cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev;
+  if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  return range(&base, &size, (CUdeviceptr)at) == CUDA_SUCCESS &&
+         size / sizeof(float) >= n && (size_t)(at - base) <= size - n * sizeof(float);
 }
 }  // namespace
 
@@ -848,7 +870,7 @@ soma_status soma_set_positions(soma_t* h, const float* src, size_t n, int src_on
   const float lim = (float)POS_LIMIT;
   unsigned flag = 0;
   SOMA_CUDA(cudaMemsetAsync(h->d_err + 2, 0, sizeof(unsigned), h->stream));
-  if (src_on_device && on_this_device(src)) {
+  if (src_on_device && readable_floats(src, n)) {
     SOMA_CUDA(launch_copy_check(src, h->pos, h->M, h->plane, lim, h->d_err + 2, h->sm_count, h->stream));
   } else {
     const cudaMemcpyKind k = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
