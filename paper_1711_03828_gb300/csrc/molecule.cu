@@ -42,6 +42,11 @@ __device__ __forceinline__ uint32_t mol_partner(uint32_t w, int k) { return (w >
 template <typename WT, uint32_t MOL_LANES, bool TOPO, bool MULTI = false>
 __device__ __forceinline__ void molecule_body(const SweepArgs& p, const TopoArgs& tp) {
   constexpr uint32_t MOL_CHAINS = 32u / MOL_LANES;   // chains of a warp
+  // The next draws during this attempt's gathers: not for the two types' one lane per
+  // molecule, whose longer partner loop has no registers left for them (16.8M particles of
+  // stars, combs, rings and diblocks, 16 cycles: 4.39 ms, in turn 4.20; with the
+  // waiting rounds below and the partner mask loaded for every attempt 4.84).
+  constexpr bool AHEAD = !TOPO || MULTI || MOL_LANES > 1u;
   extern __shared__ float sm[];
   const uint32_t N = p.g.N, N_A = p.g.N_A;
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
@@ -87,10 +92,15 @@ __device__ __forceinline__ void molecule_body(const SweepArgs& p, const TopoArgs
     float* const Z = sz + (in ? c : 0u) * N;
     const uint64_t id0 = chain * N + p.g.id_base;
     uint64_t id = id0 + q;
-    uint4 rnext = philox_rk(make_uint4((uint32_t)id, (uint32_t)(id >> 32), sweep, ctr3), p.g);
+    uint4 rnext = make_uint4(0u, 0u, 0u, 0u);
+    if (AHEAD) rnext = philox_rk(make_uint4((uint32_t)id, (uint32_t)(id >> 32), sweep, ctr3), p.g);
     for (uint32_t b = 0; b < rounds; ++b) {
-      const uint4 r = rnext;
       const uint32_t j = b * MOL_LANES + q;
+      uint4 r = rnext;
+      if (!AHEAD) {
+        id = id0 + j;
+        r = philox_rk(make_uint4((uint32_t)id, (uint32_t)(id >> 32), sweep, ctr3), p.g);
+      }
       bool pending = in && j < len;
       const uint32_t i = ((r.w & 0xFFu) * len) >> 8;
       const uint32_t pw = TOPO ? __ldg(tp.ptab + arch64 + i) : 0u;
@@ -117,12 +127,62 @@ __device__ __forceinline__ void molecule_body(const SweepArgs& p, const TopoArgs
       };
       gather();
       // the next draws (independent of the outcomes) during the gathers
-      id = id0 + j + MOL_LANES;
-      rnext = philox_rk(make_uint4((uint32_t)id, (uint32_t)(id >> 32), sweep, ctr3), p.g);
+      if (AHEAD) {
+        id = id0 + j + MOL_LANES;
+        rnext = philox_rk(make_uint4((uint32_t)id, (uint32_t)(id >> 32), sweep, ctr3), p.g);
+      }
+      const uint64_t nb = TOPO && MOL_LANES > 1u ? __ldg(tp.pmask + arch64 + i) : 0ull;
+      // the decision of an attempt whose partners are where they should be; true: moved
+      auto decide = [&]() -> bool {
+        // U = sum over bonded partners of (r - n), k partners
+        float ux = 0.f, uy = 0.f, uz = 0.f, k = 0.f;
+        if (TOPO) {
+          const uint32_t deg = pw & 63u;
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            if ((uint32_t)e < deg) {
+              const uint32_t n = mol_partner(pw, e);
+              ux += xo - X[n];
+              uy += yo - Y[n];
+              uz += zo - Z[n];
+            }
+          }
+          if (deg > 3u) {   // the partners after the third, from the full mask
+            uint64_t mk = MOL_LANES > 1u ? nb : __ldg(tp.pmask + arch64 + i);
+            mk &= mk - 1ull;
+            mk &= mk - 1ull;
+            mk &= mk - 1ull;
+            for (; mk; mk &= mk - 1ull) {
+              const uint32_t n = (uint32_t)__ffsll((long long)mk) - 1u;
+              ux += xo - X[n];
+              uy += yo - Y[n];
+              uz += zo - Z[n];
+            }
+          }
+          k = (float)deg;
+        } else {
+          if (i > 0) { ux += xo - X[i - 1]; uy += yo - Y[i - 1]; uz += zo - Z[i - 1]; k += 1.f; }
+          if (i + 1 < N) { ux += xo - X[i + 1]; uy += yo - Y[i + 1]; uz += zo - Z[i + 1]; k += 1.f; }
+        }
+        const float dEf = wn - wo;
+        const float dx = xn - xo, dy = yn - yo, dz = zn - zo;
+        const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
+        const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        const float dE = fmaf(k * K1, dd, fmaf(K2, du, dEf));
+        if (!(dE <= -log_uniform_open(r.w))) return false;
+        X[i] = xn;
+        Y[i] = yn;
+        Z[i] = zn;
+        ++my_acc;
+        return true;
+      };
+      if (MOL_LANES == 1u) {   // no other attempt to wait for
+        if (pending) decide();
+        continue;
+      }
       // earlier attempts of the group on this particle (same) or on it or a
       // bonded partner (dep), as bits of their lanes in the group
       uint32_t dep = 0u, same = 0u;
-      const uint64_t nb = TOPO ? __ldg(tp.pmask + arch64 + i) : 0ull;
 #pragma unroll
       for (uint32_t s = 0; s + 1u < MOL_LANES; ++s) {
         const uint32_t is = __shfl_sync(FULL, i, (int)(group0 + s));
@@ -135,51 +195,9 @@ __device__ __forceinline__ void molecule_body(const SweepArgs& p, const TopoArgs
       }
       uint32_t left = __ballot_sync(FULL, pending);
       while (left) {
-        const bool ready = pending && !(dep & (left >> group0));
         bool acc = false;
-        if (ready) {
-          // U = sum over bonded partners of (r - n), k partners
-          float ux = 0.f, uy = 0.f, uz = 0.f, k = 0.f;
-          if (TOPO) {
-            const uint32_t deg = pw & 63u;
-#pragma unroll
-            for (int e = 0; e < 3; ++e) {
-              if ((uint32_t)e < deg) {
-                const uint32_t n = mol_partner(pw, e);
-                ux += xo - X[n];
-                uy += yo - Y[n];
-                uz += zo - Z[n];
-              }
-            }
-            if (deg > 3u) {   // the partners after the third, from the full mask
-              uint64_t mk = nb;
-              mk &= mk - 1ull;
-              mk &= mk - 1ull;
-              mk &= mk - 1ull;
-              for (; mk; mk &= mk - 1ull) {
-                const uint32_t n = (uint32_t)__ffsll((long long)mk) - 1u;
-                ux += xo - X[n];
-                uy += yo - Y[n];
-                uz += zo - Z[n];
-              }
-            }
-            k = (float)deg;
-          } else {
-            if (i > 0) { ux += xo - X[i - 1]; uy += yo - Y[i - 1]; uz += zo - Z[i - 1]; k += 1.f; }
-            if (i + 1 < N) { ux += xo - X[i + 1]; uy += yo - Y[i + 1]; uz += zo - Z[i + 1]; k += 1.f; }
-          }
-          const float dEf = wn - wo;
-          const float dx = xn - xo, dy = yn - yo, dz = zn - zo;
-          const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
-          const float dd = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          const float dE = fmaf(k * K1, dd, fmaf(K2, du, dEf));
-          if (dE <= -log_uniform_open(r.w)) {
-            X[i] = xn;
-            Y[i] = yn;
-            Z[i] = zn;
-            ++my_acc;
-            acc = true;
-          }
+        if (pending && !(dep & (left >> group0))) {
+          acc = decide();
           pending = false;
         }
         __syncwarp();
@@ -189,6 +207,7 @@ __device__ __forceinline__ void molecule_body(const SweepArgs& p, const TopoArgs
       }
       __syncwarp();
     }
+    __syncwarp();
     // write back and count the final cells
     uint32_t ci = lane % N;
     const uint32_t step = 32u % N;
@@ -226,8 +245,11 @@ __global__ void __launch_bounds__(MOL_BLOCK, 8) sweep_molecule_kernel(const Swee
   molecule_body<WT, LANES, false>(p, TopoArgs{});
 }
 
+// One lane per molecule of n_t types: more than 64 registers, at which three types (16.8M
+// particles, 16 cycles) take 4.48 ms instead of 4.38.
 template <typename WT, uint32_t LANES, bool MULTI>
-__global__ void __launch_bounds__(MOL_BLOCK, 8) sweep_molecule_topology_kernel(const TopoArgs t) {
+__global__ void __launch_bounds__(MOL_BLOCK, MULTI && LANES == 1u ? 4 : 8)
+    sweep_molecule_topology_kernel(const TopoArgs t) {
   molecule_body<WT, LANES, true, MULTI>(t.s, t);
 }
 
