@@ -42,6 +42,14 @@ __device__ __forceinline__ void chained_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Whether this warp is one too many for its block's range [begin, begin + count) of
+// all `end` units of work, one of which goes to each warp: it leaves at once, and the
+// units go to the first warps, evenly over the SM's four schedulers, not to the ones
+// that come first (strips of 300,000 particles: up to 9 % of a cycle).
+__device__ __forceinline__ bool idle_warp(uint32_t begin, uint32_t count, uint32_t end) {
+  return (threadIdx.x >> 5) >= min(count, end - min(begin, end));
+}
+
 // Symmetric uniform (2k+1)/2^24 - 1 of the top 24 bits k of r: never 0, and
 // exact in FP32: k*2^-23 + (2^-24 - 1) is representable, and the fused
 // multiply-add rounds the exact value once.

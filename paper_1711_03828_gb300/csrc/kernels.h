@@ -46,7 +46,8 @@ struct SweepShape {
   int move;   // 0 uniform, 1 smart Monte Carlo, 2 learned
   bool learned_tc;  // learned move with the network on the tensor cores
   bool learned_umma;  // ... through tcgen05 (else warp-level mma.sync)
-  bool molecule;      // molecule-parallel iteration (one thread per chain)
+  bool molecule;      // molecule-parallel iteration
+  bool chained;       // launched with launch_chained
   int block;
   int grid;
 };

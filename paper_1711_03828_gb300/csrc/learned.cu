@@ -243,9 +243,8 @@ cudaError_t launch_sweep_learned(const SweepArgs& a, const SweepShape& s, int gr
   void* args[] = {const_cast<SweepArgs*>(&a), const_cast<void**>(&wq)};
   const void* fn = s.learned_tc ? learned_tc_kernel_ptr(s.learned_umma)
                                 : learned_kernel_ptr(s.Q, grid_dtype);
-  return s.learned_tc && !s.learned_umma
-             ? launch_chained(fn, dim3(s.grid), dim3(s.block), args, 0, st)
-             : cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, 0, st);
+  return s.chained ? launch_chained(fn, dim3(s.grid), dim3(s.block), args, 0, st)
+                   : cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, 0, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(896, 1) sweep_smc_pair_kernel(const SweepArgs 
   const uint32_t t_end = min(t_begin + chunk, n_tiles_all);
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  if (idle_warp(t_begin, chunk, n_tiles_all)) return;
   auto claim = [&]() -> uint32_t {
     uint32_t t = 0u;
     if (lane == 0) t = atomicAdd(&s_next, 1u);
@@ -200,6 +201,7 @@ __global__ void __launch_bounds__(896, 1) sweep_smc_strip_kernel(const SweepArgs
   const uint32_t item0 = blockIdx.x * chunk;
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  if (idle_warp(item0, chunk, p.n_items)) return;
   chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;

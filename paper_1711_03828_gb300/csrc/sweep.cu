@@ -20,6 +20,8 @@
 //
 // Streams: positions are loaded and stored with evict-first hints so the
 // 28 MB grid and the omega planes stay in L2.
+#include <algorithm>
+
 #include "kernels.h"
 #include "pair_body.cuh"
 #include "strip.cuh"
@@ -55,6 +57,9 @@ __global__ void __launch_bounds__(1024, 1) sweep_strip_kernel(const SweepArgs p)
   const uint32_t item0 = blockIdx.x * chunk;
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  // (a few items a block: their warps wait on latencies alone, and leaving the others
+  // before the wait measured up to 12 % slower)
+  if (chunk >= 8u && idle_warp(item0, chunk, p.n_items)) return;
   chained_begin();
   const unsigned long long s64 = *p.d_sweep;
   const uint32_t sweep = (uint32_t)s64;
@@ -188,6 +193,7 @@ __global__ void __launch_bounds__(1024, 1) sweep_pair_kernel(const SweepArgs p) 
   const uint32_t t_end = min(t_begin + chunk, n_tiles_all);
   if (threadIdx.x == 0) s_next = 0u;
   __syncthreads();
+  if (idle_warp(t_begin, chunk, n_tiles_all)) return;
   auto claim = [&]() -> uint32_t {
     uint32_t t = 0u;
     if (lane == 0) t = atomicAdd(&s_next, 1u);
@@ -289,18 +295,27 @@ static const void* sweep_kernel_ptr(const SweepShape& s, int grid_dtype, bool mi
 }
 
 // Chains per work item of the strip kernels: C chains of U units take
-// ceil(C U / 32) strips (and a draw per chain for the set orders, about a
-// sixth of a strip), n/C items go round `warps` warps.  The C of the lowest
-// time under that count; at most 12 strips (or one chain), so that the warps
-// of a block stay near one another in space.
-static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t warps) {
+// ceil(C U / 32) strips, and the n/C items go to the warps of one block per SM.  The C
+// of the lowest cost: a block's items times their strips (what its warps issue; each
+// item a draw per chain and its last strip partly empty besides), and per round of
+// warps the latency of one item's strips, which the others hide once.  Without the
+// latency, one round of many short items looked as good as one of few full ones:
+// 16 cycles of 65,536 particles, N = 5, took 161 us in items of 3 chains (9 of 32 lanes)
+// and take 124 in items of 10.  Over 286 systems of N = 3 to 256 and 8,000 to 16M
+// particles every C of at most 32 strips was timed: the one chosen here takes 1.7 %
+// longer than the best on average, the one of fewest rounds alone 6.7 %.
+constexpr uint32_t STRIPS_MAX = 32;
+constexpr double ITEM_COST = 0.5, ROUND_COST = 6.0;   // strips; items
+
+static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t sms, uint64_t warps) {
   uint32_t best = 1;
   double least = 0.0;
   for (uint32_t C = 1; C <= 32u; ++C) {
     const uint32_t strips = (C * U + 31u) / 32u;
-    if (C > 1u && strips > 12u) break;
-    const uint64_t items = (n + C - 1u) / C;
-    const double cost = (double)((items + warps - 1u) / warps) * ((double)strips + 1.0 / 6.0);
+    if (C > 1u && strips > STRIPS_MAX) break;
+    const uint64_t items = (n + C - 1u) / C, per = (items + sms - 1u) / sms;
+    const uint64_t rounds = (per + warps - 1u) / warps;
+    const double cost = ((double)per + ROUND_COST * (double)rounds) * ((double)strips + ITEM_COST);
     if (C == 1u || cost < least) {
       least = cost;
       best = C;
@@ -308,6 +323,11 @@ static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t warps) {
   }
   return best;
 }
+
+// Most rounds of a block's warps that are made even by launching fewer warps: 76
+// tiles per SM (734,000 particles, 16 cycles) take 211 us in 3 rounds of 26 warps, 227
+// with 32, of which 12 work in the last round.
+constexpr uint64_t EVEN_ROUNDS = 8;
 
 SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bool learned_fp32,
                        bool learned_umma, bool molecule) {
@@ -331,35 +351,56 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   s.strip = !s.pair || (move == 1 && (s.big || s.G * s.units < 32u));
   if (move == 2 || (molecule && move == 0)) s.strip = false;
   s.block = 256;
+  s.chained = false;
+  bool one_per_sm = false;
   if (move == 2 && s.pair && !s.big && !learned_fp32) {
     s.learned_tc = true;
     s.learned_umma = learned_umma;
-    s.block = learned_umma ? 128 : 512;   // one block of 12 warps per SM (mma.sync)
+    one_per_sm = !learned_umma;
+    s.block = learned_umma ? 128 : 512;   // 16 warps (mma.sync, learned_tc.cu)
   } else if (molecule && move == 0) {
     s.molecule = true;
     s.block = MOL_BLOCK;
   } else if (move != 2) {
-    // one block per SM: 32 warps in 64 registers without spills for uniform moves
-    // (16 cycles of 134M particles with 24 warps 16.56 ms, 28 16.42, 32 16.22; thin
-    // film 2.61, 2.46, 2.43), 28 for smart Monte Carlo (smc.cu)
+    // 32 warps in 64 registers without spills for uniform moves (16 cycles of 134M
+    // particles with 24 warps 16.56 ms, 28 16.42, 32 16.22; thin film 2.61, 2.46,
+    // 2.43), 28 for smart Monte Carlo (smc.cu)
+    one_per_sm = true;
     s.block = move == 1 ? 896 : 1024;
   }
-  s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count * (s.block / 32)) : 0u;
+  s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count, (uint64_t)s.block / 32) : 0u;
   s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
-  const void* fn = s.learned_tc ? learned_tc_kernel_ptr(s.learned_umma)
-                                : sweep_kernel_ptr(s, grid_dtype, false);
   if (s.molecule) {
     s.grid = molecule_grid(n_chains, N, grid_dtype, sm_count);
     return s;
   }
+  if (one_per_sm) {
+    // over all SMs, however little work there is: 16 cycles of force-biased moves of
+    // 65,536 particles (1,024 tiles) 150 us on the 37 SMs that full blocks fill, 136 on all
+    const uint64_t work = s.strip ? s.n_items : s.n_tiles;
+    s.grid = (int)(work < (uint64_t)sm_count ? work : (uint64_t)sm_count);
+    const uint64_t per = (work + (uint64_t)s.grid - 1) / (uint64_t)s.grid;
+    const uint64_t warps = (uint64_t)s.block / 32, rounds = (per + warps - 1) / warps;
+    if (rounds > 1u && rounds <= EVEN_ROUNDS) s.block = 32 * (int)((per + rounds - 1) / rounds);
+    s.chained = true;
+    if (s.learned_tc && rounds == 1u) {
+      // no more warps than tiles (four to load the fragments): two blocks then fit on
+      // an SM, and where they are more than a few warps the next cycle's, set up ahead,
+      // would share SMs unevenly with this one's (65,536 particles, 16 cycles: 16 warps
+      // 217 us, as many as tiles 198 set up ahead, 178 not; 4,096: 16 warps 140, four 141
+      // set up ahead, 149 not)
+      s.block = 32 * (int)std::max<uint64_t>(4u, per);
+      s.chained = s.block <= 128 || s.block > 256;
+    }
+    return s;
+  }
+  const void* fn = s.learned_tc ? learned_tc_kernel_ptr(s.learned_umma)
+                                : sweep_kernel_ptr(s, grid_dtype, false);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, 0);
   if (per_sm < 1) per_sm = 1;
   const uint64_t warps_per_block = (uint64_t)s.block / 32;
-  // strips and learned tiles are spread over all SMs, however few they are
-  const uint64_t need = s.strip    ? s.n_items
-                      : s.learned_tc && !s.learned_umma ? s.n_tiles
-                                   : (s.n_tiles + warps_per_block - 1) / warps_per_block;
+  const uint64_t need = (s.n_tiles + warps_per_block - 1) / warps_per_block;
   const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
   s.grid = (int)(need < cap ? need : cap);
   if (s.grid < 1) s.grid = 1;
@@ -372,8 +413,8 @@ cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int gr
   const void* fn = s.molecule ? molecule_kernel(a.g.n_chains, a.g.N, grid_dtype, sm_count, &smem)
                               : sweep_kernel_ptr(s, grid_dtype, a.seq != nullptr);
   void* args[] = {const_cast<SweepArgs*>(&a)};
-  return s.molecule ? cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st)
-                    : launch_chained(fn, dim3(s.grid), dim3(s.block), args, smem, st);
+  return s.chained ? launch_chained(fn, dim3(s.grid), dim3(s.block), args, smem, st)
+                   : cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st);
 }
 
 }  // namespace soma
