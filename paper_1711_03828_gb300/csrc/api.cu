@@ -344,6 +344,7 @@ SweepArgs sweep_args(soma_t* h, const SweepShape& sh) {
   s.strip_units = sh.units;
   s.strip_chains = sh.chains;
   s.n_items = (uint32_t)sh.n_items;
+  s.strip_order = s.strip_odd = 0u;
   s.set_order_random = h->desc.set_order == SOMA_SET_ORDER_RANDOM;
   const double A = h->a64 * h->a64 / 6.0;
   s.smc_A = (float)A;

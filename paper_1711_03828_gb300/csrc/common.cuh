@@ -235,9 +235,11 @@ struct SweepArgs {
   uint64_t n_tiles;
   uint64_t full_tiles;      // tiles holding G chains
   uint32_t last_rows;       // particles in the last, partial tile (0: none)
-  uint32_t strip_units;     // strip layout: units per chain, chains per item, items
+  uint32_t strip_units;     // strip layout: units per chain, chains per item, items,
   uint32_t strip_chains;
   uint32_t n_items;
+  uint32_t strip_order;     // set-order bits of a fixed order, not those of the last chain
+  uint32_t strip_odd;       // (single particles in pairs, an odd number of them)
   int set_order_random;
   // smart Monte Carlo: A = a^2/6, sqrt(2A), 1/(4A)
   float smc_A, smc_s2A, smc_inv4A;

@@ -84,7 +84,8 @@ struct StripWalk {
     strips = (n_ch * U + 31u) / 32u;
     c = (uint32_t)lane / U;
     k = (uint32_t)lane - c * U;
-    bits = 0u;
+    bits = p.strip_order;
+    if (p.strip_odd && rem <= (IDX)p.strip_chains) bits ^= 1u << (n_ch - 1u);
     if (p.set_order_random) {   // bit 0 of word 3 of the move draw of each chain's particle 0
       const uint64_t m = (uint64_t)(chain0 + lane) * p.g.N + p.g.id_base;
       const uint4 w = philox_rk(make_uint4((uint32_t)m, (uint32_t)(m >> 32), sweep, ctr3), p.g);

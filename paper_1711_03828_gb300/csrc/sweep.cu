@@ -344,7 +344,7 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   s.pair = (s.Q == 1) && (N % 2 == 0);
   s.big = n_chains * N >= (1ull << 32) || s.n_tiles >= (1ull << 31);
   s.wide = g.nx > 1 && g.ny > 1 && g.nz > 1;
-  s.units = N / 2u + 1u;
+  s.units = N == 1u ? 1u : N / 2u + 1u;
   // Uniform moves of even N <= 64 run in pair tiles.  Smart Monte Carlo moves
   // do where the tiles hold at least as many particles per slot as the strips
   // (G N of 64 slots against N of 2 U) and the indices fit 32 bits.
@@ -368,8 +368,9 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
     one_per_sm = true;
     s.block = move == 1 ? 896 : 1024;
   }
-  s.chains = s.strip ? strip_chains(n_chains, s.units, (uint64_t)sm_count, (uint64_t)s.block / 32) : 0u;
-  s.n_items = s.strip ? (n_chains + s.chains - 1) / s.chains : 0u;
+  const uint64_t walked = N == 1u ? (n_chains + 1u) / 2u : n_chains;   // see paired_singles
+  s.chains = s.strip ? strip_chains(walked, s.units, (uint64_t)sm_count, (uint64_t)s.block / 32) : 0u;
+  s.n_items = s.strip ? (walked + s.chains - 1) / s.chains : 0u;
   if (s.molecule) {
     s.grid = molecule_grid(n_chains, N, grid_dtype, sm_count);
     return s;
@@ -407,12 +408,29 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
   return s;
 }
 
+// Chains of one particle have no bonds (K_b = 0) and no set order to keep: two of them
+// walk as one chain of two, which fills a unit; one alone leaves a slot of it empty (2M
+// single particles, 16 cycles: 770 and 1017 us one by one, 459 and 589 in pairs, uniform
+// and force-biased).  The one left over of an odd number is the even particle of a pair
+// whose even ones come first, a unit without its odd one.
+static SweepArgs paired_singles(const SweepArgs& a) {
+  SweepArgs b = a;
+  b.g.N = 2u;
+  b.g.N_A = 2u * a.g.N_A;
+  b.g.n_chains = (a.g.n_chains + 1u) / 2u;
+  b.set_order_random = 0;
+  b.strip_order = FULL;
+  b.strip_odd = (uint32_t)(a.g.n_chains & 1u);
+  return b;
+}
+
 cudaError_t launch_sweep_uniform(const SweepArgs& a, const SweepShape& s, int grid_dtype,
                                  int sm_count, cudaStream_t st) {
   size_t smem = 0;
   const void* fn = s.molecule ? molecule_kernel(a.g.n_chains, a.g.N, grid_dtype, sm_count, &smem)
                               : sweep_kernel_ptr(s, grid_dtype, a.seq != nullptr);
-  void* args[] = {const_cast<SweepArgs*>(&a)};
+  const SweepArgs b = s.strip && a.g.N == 1u ? paired_singles(a) : a;
+  void* args[] = {const_cast<SweepArgs*>(&b)};
   return s.chained ? launch_chained(fn, dim3(s.grid), dim3(s.block), args, smem, st)
                    : cudaLaunchKernel(fn, dim3(s.grid), dim3(s.block), args, smem, st);
 }

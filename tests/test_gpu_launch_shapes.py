@@ -1,8 +1,9 @@
 """Launch shapes of the one-block-per-SM sweeps at the edges of their rules: less
 work than SMs, one unit a block, one round of warps exactly and one unit more (a
 block then has fewer warps), the uniform strips' blocks of fewer than eight items
-and more, the learned sweep's of four warps, five to eight and more.  One cycle
-against the oracle, and one call of many cycles against as many of one."""
+and more, the learned sweep's of four warps, five to eight and more, and chains of
+one particle, which strips take in pairs.  One cycle against the oracle, and one call
+of many cycles against as many of one."""
 import numpy as np
 import pytest
 
@@ -54,3 +55,24 @@ def test_strips(cuda_device, move, N, n):
 @pytest.mark.parametrize("tiles", [4 * SMS, 4 * SMS + 1, 8 * SMS + 1, 16 * SMS + 1])
 def test_learned_tiles(cuda_device, tiles):
     learned_one_cycle(cuda_device, 64, tiles, GRID, BOX, 0)
+
+
+# two single particles walk as one chain: an odd one left over, alone and past a strip
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 701, 64 * SMS + 1])
+def test_single_particles(cuda_device, n):
+    _compare(1, n, MOVE_UNIFORM)
+
+
+@pytest.mark.parametrize("f", [0.4, 0.6])     # all B, all A
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 701, 64 * SMS + 1])
+def test_single_particles_force_biased(cuda_device, n, f):
+    """Against the architecture sweep of molecules of one particle."""
+    d = SystemDesc(n_chains=n, N=1, f=f, box_Re=BOX, grid=GRID, chiN=25.0, kappaN=30.0, seed=23, move=MOVE_SMC)
+    strips, molecules = System(d), System(d)
+    molecules.set_architectures([int(f < 0.5)], np.zeros(n, np.uint8))
+    for cycles in (1, 18):
+        strips.sweep(cycles)
+        molecules.sweep(cycles)
+        np.testing.assert_array_equal(strips.get_positions(), molecules.get_positions())
+        np.testing.assert_array_equal(strips.get_density(), molecules.get_density())
+    assert 0 < strips.observables()["accepted"] == molecules.observables()["accepted"]
