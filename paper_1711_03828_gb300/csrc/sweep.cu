@@ -298,14 +298,17 @@ static const void* sweep_kernel_ptr(const SweepShape& s, int grid_dtype, bool mi
 // ceil(C U / 32) strips, and the n/C items go to the warps of one block per SM.  The C
 // of the lowest cost: a block's items times their strips (what its warps issue; each
 // item a draw per chain and its last strip partly empty besides), and per round of
-// warps the latency of one item's strips, which the others hide once.  Without the
-// latency, one round of many short items looked as good as one of few full ones:
-// 16 cycles of 65,536 particles, N = 5, took 161 us in items of 3 chains (9 of 32 lanes)
-// and take 124 in items of 10.  Over 286 systems of N = 3 to 256 and 8,000 to 16M
-// particles every C of at most 32 strips was timed: the one chosen here takes 1.7 %
-// longer than the best on average, the one of fewest rounds alone 6.7 %.
+// warps the latency of one item's strips, which the others hide once; and the more
+// strips an item has, the further apart in space a block's warps work (their field
+// values repeat less in L1).  Without the latency, one round of many short items looked
+// as good as one of few full ones: 16 cycles of 65,536 particles, N = 5, took 161 us in
+// items of 3 chains (9 of 32 lanes) and take 124 in items of 10.  Without the distance,
+// the thin film (N = 100, 16.5M) took 2.48 ms in items of 18 chains, 2.43 in items of 5.
+// Over 286 systems of N = 3 to 256 and 8,000 to 16M particles every C of at most 32
+// strips was timed: the one chosen here takes 1.0 % longer than the best on average,
+// the one of fewest rounds alone 7.1 %.
 constexpr uint32_t STRIPS_MAX = 32;
-constexpr double ITEM_COST = 0.5, ROUND_COST = 6.0;   // strips; items
+constexpr double ITEM_COST = 1.5, SPREAD_COST = 0.015, ROUND_COST = 8.0;   // strips; items
 
 static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t sms, uint64_t warps) {
   uint32_t best = 1;
@@ -315,7 +318,8 @@ static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t sms, uint64_t warp
     if (C > 1u && strips > STRIPS_MAX) break;
     const uint64_t items = (n + C - 1u) / C, per = (items + sms - 1u) / sms;
     const uint64_t rounds = (per + warps - 1u) / warps;
-    const double cost = ((double)per + ROUND_COST * (double)rounds) * ((double)strips + ITEM_COST);
+    const double cost = ((double)per + ROUND_COST * (double)rounds) *
+                        ((double)strips + ITEM_COST + SPREAD_COST * strips * strips);
     if (C == 1u || cost < least) {
       least = cost;
       best = C;
@@ -326,7 +330,9 @@ static uint32_t strip_chains(uint64_t n, uint32_t U, uint64_t sms, uint64_t warp
 
 // Most rounds of a block's warps that are made even by launching fewer warps: 76
 // tiles per SM (734,000 particles, 16 cycles) take 211 us in 3 rounds of 26 warps, 227
-// with 32, of which 12 work in the last round.
+// with 32, of which 12 work in the last round.  Where more than half of them would work
+// there, all are better (the thin film's 217 items in 7 rounds: 2.44 ms with 31 warps,
+// 2.43 with 32).
 constexpr uint64_t EVEN_ROUNDS = 8;
 
 SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bool learned_fp32,
@@ -382,7 +388,8 @@ SweepShape sweep_shape(const Geom& g, int sm_count, int grid_dtype, int move, bo
     s.grid = (int)(work < (uint64_t)sm_count ? work : (uint64_t)sm_count);
     const uint64_t per = (work + (uint64_t)s.grid - 1) / (uint64_t)s.grid;
     const uint64_t warps = (uint64_t)s.block / 32, rounds = (per + warps - 1) / warps;
-    if (rounds > 1u && rounds <= EVEN_ROUNDS) s.block = 32 * (int)((per + rounds - 1) / rounds);
+    if (rounds > 1u && rounds <= EVEN_ROUNDS && 2u * (rounds * warps - per) >= warps)
+      s.block = 32 * (int)((per + rounds - 1) / rounds);
     s.chained = true;
     if (s.learned_tc && rounds == 1u) {
       // no more warps than tiles (four to load the fragments): two blocks then fit on
