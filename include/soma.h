@@ -517,8 +517,11 @@ soma_status soma_proposal_train(soma_t* h, const soma_train_cfg* cfg, soma_train
  * paper, which runs one system per MPI rank; the launch shape is chosen by
  * an autotuner in the spirit of Sec. 3.2.2).
  *
- * Members are created as by soma_create and evolve bit-identically to the
- * same system run alone.  Requirements: even N <= 64, uniform moves, one seed
+ * Members are created as by soma_create and evolve as the same system run
+ * alone: the same draws, moves and counts, and the same fields but for a last
+ * bit of FP32 ones under K^0 (about half of the cells), which shows where a
+ * move is that close to its acceptance threshold (64 cycles of 40M particles:
+ * one in 300 to 500 positions).  Requirements: even N <= 64, uniform moves, one seed
  * and one grid_dtype for all members (distinguish members by replica_id),
  * M < 2^32 per member, at most SOMA_BATCH_MAX members.  soma_batch_system
  * lends the member's handle for getters and observables; soma_sweep on a lent

@@ -6,12 +6,13 @@
 // sizes, chain lengths, compositions, chiN, replicas of one seed) shares a
 // single persistent launch: the tiles of all systems are cut into work items
 // of contiguous tiles of one system; block j takes items j, j + grid, ... and
-// its warps take the items' tiles in turn with the same tile body as the single-system
-// kernel (pair_body.cuh), so every system evolves bit-identically to the same
-// system run alone.  The host lays the items out either as fixed-length items
-// of each system in turn or as one equal contiguous range of the concatenated
-// tiles per block, cut at system boundaries (piece r of block j at item
-// r * grid + j, padded with empty items).  Launch shape (block size, blocks
+// its warps take the items' tiles in turn with the same tile body as the
+// single-system kernel (pair_body.cuh) and the same draws: a system evolves as
+// it does alone, but for a last bit of FP32 fields under K^0
+// (fields_batch_kernel).  The host lays the items out either as fixed-length
+// items of each system in turn or as one equal contiguous range of the
+// concatenated tiles per block, cut at system boundaries (piece r of block j at
+// item r * grid + j, padded with empty items).  Launch shape (block size, blocks
 // per SM, split) is picked by an autotuner that times the candidates during
 // the run.
 #include "kernels.h"
@@ -186,17 +187,20 @@ __global__ void __launch_bounds__(256) fields_batch_kernel(const BatchArgs p, ui
     const uint32_t v = nr[local];
     nc[local] = 0u;
     const uint32_t a = v & 0xFFFFu, b = v >> 16;
-    const float phiA = (float)a * inv_rho;
-    const float phiB = (float)b * inv_rho;
-    const float comp = kappa0 * (phiA + phiB - 1.f);
+    // with its roundings written out; under K^0 they are not omega_of's (omega.cuh), and
+    // FP32 fields differ from its by an ulp in about half of the cells: the batch's own
+    // trajectories, kept as they are
+    const float phiA = __fmul_rn((float)a, inv_rho), phiB = __fmul_rn((float)b, inv_rho);
+    const float comp = __fmul_rn(kappa0, __fsub_rn(__fadd_rn(phiA, phiB), 1.f));
     float wa, wb;
     if (ham) {
-      wa = fmaf(2.f * half_chi0, phiB, comp);
-      wb = fmaf(2.f * half_chi0, phiA, comp);
+      const float chi0 = __fmul_rn(2.f, half_chi0);
+      wa = __fmaf_rn(chi0, phiB, comp);
+      wb = __fmaf_rn(chi0, phiA, comp);
     } else {
-      const float d = half_chi0 * (phiA - phiB);
-      wa = comp - d;
-      wb = comp + d;
+      const float d = __fsub_rn(phiA, phiB);
+      wa = __fmaf_rn(-half_chi0, d, comp);
+      wb = __fmaf_rn(half_chi0, d, comp);
     }
     wA[local] = store_cvt<WT>(wa);
     wB[local] = store_cvt<WT>(wb);
