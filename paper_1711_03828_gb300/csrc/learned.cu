@@ -390,10 +390,10 @@ __global__ void __launch_bounds__(GRAD_T) esjd_grad_kernel(TrainArgs t) {
   const Geom& g = t.g;
   const uint32_t N = g.N;
   GradAcc A = {};
-  for (uint32_t s0 = blockIdx.x * GRAD_S; s0 < t.n; s0 += gridDim.x * GRAD_S) {
+  for (uint64_t s0 = (uint64_t)blockIdx.x * GRAD_S; s0 < t.n; s0 += (uint64_t)gridDim.x * GRAD_S) {
     // a lane past the batch repeats its last sample with zero gradients
-    const bool valid = s0 + (uint32_t)lane < t.n;
-    const uint32_t b = valid ? s0 + (uint32_t)lane : t.n - 1u;
+    const bool valid = s0 + (uint64_t)lane < t.n;
+    const uint64_t b = valid ? s0 + (uint64_t)lane : t.n - 1u;
     uint64_t chain;
     uint32_t i;
     float xi[3];
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(256) train_sums_kernel(const float* __restrict
                                                          uint32_t n, double* __restrict__ part) {
   __shared__ double sh[2 * 32];
   double v[2] = {0.0, 0.0};
-  for (uint32_t b = blockIdx.x * 256u + threadIdx.x; b < n; b += gridDim.x * 256u) {
+  for (uint64_t b = blockIdx.x * 256u + threadIdx.x; b < n; b += gridDim.x * 256u) {
     const float l = log_alpha[b];
     v[0] += (double)J[b];
     v[1] += l >= 0.f ? 1.0 : exp((double)l);
