@@ -76,7 +76,10 @@ struct ResidentArgs {
 // Largest system of the resident sweep, in tiles of 64 slots per SM: two rounds of
 // 32 warps.  Resident against two kernels a cycle in long calls: 27 tiles per SM 7.4
 // and 9.3 us, 40 9.1 and 11.1, 61 11.0 and 11.9, 91 14.1 and 14.5 (16 cycles 234 and
-// 229), 121 16.8 and 16.6.
+// 229), 121 16.8 and 16.6.  That is for a system alone: its blocks hold their SMs for all
+// cycles, and several systems on their own streams, which two kernels a cycle let in
+// turn, wait for one another (four of 32,768 particles 237 us for 32 cycles, with two
+// kernels 305; of 131,072 435 and 406; of 300,000 998 and 678).
 constexpr uint64_t RESIDENT_TILES_PER_SM = 64;
 // Fewest cycles of a call that take it: two, and one more per 16 tiles per SM.  Its
 // launch and last field update cost what some cycles gain; calls back to back,

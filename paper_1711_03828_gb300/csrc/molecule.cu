@@ -255,11 +255,18 @@ __global__ void __launch_bounds__(MOL_BLOCK, MULTI && LANES == 1u ? 4 : 8)
 
 // Lanes per chain.  Four where the chains would give each SM fewer than four
 // warps at one lane each (the attempts' latencies, not the instructions, are the
-// time: 8,192 chains of 32, 26.4 us a cycle with one thread per chain, 24.7 / 17.8 /
-// 14.5 with 1 / 2 / 4 lanes); two for long chains, whose staging leaves few warps
-// on an SM at one lane each (67M particles of N = 64: 1627, 1506 / 1070 / 1173 us);
-// else one (134M of N = 32: 1984, 1871 / 2612 / 2424 us). The line: 67M
-// particles of N = 40, 1111 / 1159 us; of N = 48, 1187 / 1145.
+// time); two for long chains, whose staging leaves few warps on an SM at one lane
+// each; else one.  us a cycle with 1 / 2 / 4 lanes:
+//   chains     8,192             19,000            28,000            65,536
+//   N = 16     14.0 12.5 11.0    14.8 14.0 13.3    16.5 16.3 16.4    25.7 24.1 28.6
+//   N = 32     21.8 18.1 14.9    23.2 22.1 19.5    25.7 24.8 24.0    36.6 40.3 44.8
+//   N = 44     28.0 22.6 18.0    29.2 27.1 23.7    33.6 31.0 29.4    66.6 54.8 57.8
+//   N = 64     37.8 28.7 22.4    39.7 34.3 30.9    44.9 38.9 38.8    85.6 80.1 77.8
+//   262,144 chains of 8 33 43 58, 16 74 72 92, 32 127 142 160, 44 217 195 212, 64 339 278 294
+// (stars, combs and rings of 32: 27.1 25.6 18.5, 27.8 28.8 22.5, at 30,000 32.5 34.8
+// 30.1, 42.5 47.1 55.2).  So both lines lie a little to one side of where the times
+// cross: four lanes are as good as one up to about 30,000 chains (the line: 19,456 on
+// 152 SMs), and two as good as one from N = 36 to 42 (the line: 44).
 constexpr uint32_t MOL_ONE_LANE_N = 44;   // longest chains of one lane
 constexpr uint32_t MOL_N = 256;           // longest chains
 uint32_t molecule_lanes(uint64_t n_chains, uint32_t N, int sm_count) {
